@@ -14,6 +14,8 @@
 // Buffers ping-pong between the output and the caller's scratch so that the
 // last pass lands in the output.  The order-preserving key map is applied
 // when the tile sort loads the input and undone when the last pass stores.
+// Large sorts (radix_fits) are done by digit passes instead (radix.cu): the
+// same result in fewer passes over the array.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -24,6 +26,7 @@
 
 #include "nsort.h"
 #include "nsort_testing.h"
+#include "launch.h"
 #include "nsort_internal.h"
 #include "sort_device.cuh"
 #include "tma_device.cuh"
@@ -1566,37 +1569,6 @@ Plan make_plan(int kind, uint64_t n, int dtype) {
   return p;
 }
 
-// Launches a kernel with programmatic stream serialisation: the launch is
-// processed while the previous kernel of the stream still runs and its CTAs
-// start as soon as that kernel completes, which hides the launch latency
-// between the dependent kernels of a sort (about 20% of a 2^20-key sort, 1%
-// at 2^28).  Every kernel so launched calls pdl_wait() before it reads or
-// writes anything the previous kernels touch.  NSORT_NO_PDL=1 in the
-// environment selects plain launches.
-static bool pdl_enabled() {
-  static const bool on = [] {
-    const char *e = getenv("NSORT_NO_PDL");
-    return !(e && e[0] == '1');
-  }();
-  return on;
-}
-
-template <typename... KArgs, typename... Args>
-static void launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem,
-                       cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
 static int launch_status(const char *what) {
   const cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) return NSORT_OK;
@@ -1968,6 +1940,7 @@ static void launch_merge_staged64(const uint64_t *src, uint64_t *dst, int64_t n,
 int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void *tmp,
                      cudaStream_t st) {
   const Plan p = make_plan(NSORT_KIND_KEYS, (uint64_t)n, dt);
+  if (radix_fits(p, false, 8)) return radix_sort_keys64(p, in, out, dt, tmp, st);
   char *t = static_cast<char *>(tmp);
   uint64_t *bufs[2] = {out, p.merge_passes ? reinterpret_cast<uint64_t *>(t + p.keys_off) : nullptr};
   int64_t *split = p.merge_passes ? reinterpret_cast<int64_t *>(t + p.split_off) : nullptr;
@@ -2005,6 +1978,8 @@ int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void 
 int sort_keys_impl(const uint32_t *in, uint32_t *out, int64_t n, int dt, void *tmp,
                    cudaStream_t st) {
   const Plan p = make_plan(NSORT_KIND_KEYS, (uint64_t)n);
+  if (p.merge4_passes == 0 && radix_fits(p, false, 4))
+    return radix_sort_keys(p, in, out, dt, tmp, st);
   char *t = static_cast<char *>(tmp);
   uint32_t *bufs[2] = {out, p.merge_passes ? reinterpret_cast<uint32_t *>(t + p.keys_off) : nullptr};
   int64_t *split = p.merge_passes ? reinterpret_cast<int64_t *>(t + p.split_off) : nullptr;
@@ -2072,9 +2047,13 @@ template <typename V>
 static int sort_pairs_typed(const uint32_t *kin, const V *vin, uint32_t *kout, V *vout, int64_t n,
                             int dt, void *tmp, cudaStream_t st) {
   constexpr bool V64 = sizeof(V) == 8;
+  const Plan p = make_plan(V64 ? NSORT_KIND_PAIRS64 : NSORT_KIND_PAIRS, (uint64_t)n);
+  if (radix_fits(p, true, 4)) {
+    if constexpr (V64) return radix_sort_pairs64(p, kin, vin, kout, vout, dt, tmp, st);
+    else return radix_sort_pairs(p, kin, vin, kout, vout, dt, tmp, st);
+  }
   int rc = ensure_pairs_smem_attr<V>();
   if (rc != NSORT_OK) return rc;
-  const Plan p = make_plan(V64 ? NSORT_KIND_PAIRS64 : NSORT_KIND_PAIRS, (uint64_t)n);
   char *t = static_cast<char *>(tmp);
   uint32_t *kb[2] = {kout, p.merge_passes ? reinterpret_cast<uint32_t *>(t + p.keys_off) : nullptr};
   V *vb[2] = {vout, p.merge_passes ? reinterpret_cast<V *>(t + p.vals_off) : nullptr};

@@ -18,7 +18,8 @@ const char *const kKernelNames[] = {"tile_sort_keys", "tile_sort_pairs", "partit
                                     "merge_keys",     "merge_pairs",     "segmented_bin",
                                     "segmented_sort", "segmented_merge", "segmented_copy",
                                     "tile_sort_keys64", "merge_keys64",
-                                    "sample_merge",   "merge4_bounds",   "merge4_keys"};
+                                    "sample_merge",   "merge4_bounds",   "merge4_keys",
+                                    "radix_histogram", "radix_pass"};
 constexpr int kNumKernels = sizeof(kKernelNames) / sizeof(kKernelNames[0]);
 
 struct Rec {
