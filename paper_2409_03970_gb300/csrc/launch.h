@@ -22,7 +22,8 @@ inline bool pdl_enabled() {
   return on;
 }
 
-template <typename... KArgs, typename... Args>
+// CLUSTER: CTAs of a thread-block cluster.
+template <int CLUSTER = 1, typename... KArgs, typename... Args>
 void launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem,
                 cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
@@ -30,11 +31,14 @@ void launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t 
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = CLUSTER;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CLUSTER > 1 ? 2 : 1;
   cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 

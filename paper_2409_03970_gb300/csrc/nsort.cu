@@ -14,8 +14,8 @@
 // Buffers ping-pong between the output and the caller's scratch so that the
 // last pass lands in the output.  The order-preserving key map is applied
 // when the tile sort loads the input and undone when the last pass stores.
-// Large sorts (radix_fits) are done by digit passes instead (radix.cu): the
-// same result in fewer passes over the array.
+// Most sorts of more than a tile are done by digit passes instead (radix.cu):
+// the same result in fewer passes over the array.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -1940,7 +1940,9 @@ static void launch_merge_staged64(const uint64_t *src, uint64_t *dst, int64_t n,
 int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void *tmp,
                      cudaStream_t st) {
   const Plan p = make_plan(NSORT_KIND_KEYS, (uint64_t)n, dt);
-  if (radix_fits(p, false, 8)) return radix_sort_keys64(p, in, out, dt, tmp, st);
+  bool sorted = false;
+  int rc = radix_sort_keys64(p, &sorted, in, out, dt, tmp, st);
+  if (sorted || rc != NSORT_OK) return rc;
   char *t = static_cast<char *>(tmp);
   uint64_t *bufs[2] = {out, p.merge_passes ? reinterpret_cast<uint64_t *>(t + p.keys_off) : nullptr};
   int64_t *split = p.merge_passes ? reinterpret_cast<int64_t *>(t + p.split_off) : nullptr;
@@ -1956,7 +1958,7 @@ int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void 
     launch_tile_sort_keys64(in, bufs[cur], n, dt, p.merge_passes == 0, (unsigned)tiles,
                             tma ? samp : nullptr, st);
   }
-  int rc = launch_status("tile_sort_keys64");
+  rc = launch_status("tile_sort_keys64");
   for (int pass = 0; rc == NSORT_OK && pass < p.merge_passes; ++pass) {
     const int64_t run = (int64_t)p.sort_tile << pass;
     const bool last = pass == p.merge_passes - 1;
@@ -1978,8 +1980,12 @@ int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void 
 int sort_keys_impl(const uint32_t *in, uint32_t *out, int64_t n, int dt, void *tmp,
                    cudaStream_t st) {
   const Plan p = make_plan(NSORT_KIND_KEYS, (uint64_t)n);
-  if (p.merge4_passes == 0 && radix_fits(p, false, 4))
-    return radix_sort_keys(p, in, out, dt, tmp, st);
+  int rc = NSORT_OK;
+  if (p.merge4_passes == 0) {
+    bool sorted = false;
+    rc = radix_sort_keys(p, &sorted, in, out, dt, tmp, st);
+    if (sorted || rc != NSORT_OK) return rc;
+  }
   char *t = static_cast<char *>(tmp);
   uint32_t *bufs[2] = {out, p.merge_passes ? reinterpret_cast<uint32_t *>(t + p.keys_off) : nullptr};
   int64_t *split = p.merge_passes ? reinterpret_cast<int64_t *>(t + p.split_off) : nullptr;
@@ -2003,7 +2009,7 @@ int sort_keys_impl(const uint32_t *in, uint32_t *out, int64_t n, int dt, void *t
       launch_tile_sort_keys(in, bufs[cur], n, dt, p.merge_passes == 0, (unsigned)tiles,
                             tma ? samp : nullptr, st);
   }
-  int rc = launch_status("tile_sort_keys");
+  rc = launch_status("tile_sort_keys");
   int64_t run = p.sort_tile;
   for (int pass = 0; rc == NSORT_OK && pass < npass; ++pass) {
     const bool last = pass == npass - 1;
@@ -2048,11 +2054,12 @@ static int sort_pairs_typed(const uint32_t *kin, const V *vin, uint32_t *kout, V
                             int dt, void *tmp, cudaStream_t st) {
   constexpr bool V64 = sizeof(V) == 8;
   const Plan p = make_plan(V64 ? NSORT_KIND_PAIRS64 : NSORT_KIND_PAIRS, (uint64_t)n);
-  if (radix_fits(p, true, 4)) {
-    if constexpr (V64) return radix_sort_pairs64(p, kin, vin, kout, vout, dt, tmp, st);
-    else return radix_sort_pairs(p, kin, vin, kout, vout, dt, tmp, st);
-  }
-  int rc = ensure_pairs_smem_attr<V>();
+  bool sorted = false;
+  int rc;
+  if constexpr (V64) rc = radix_sort_pairs64(p, &sorted, kin, vin, kout, vout, dt, tmp, st);
+  else rc = radix_sort_pairs(p, &sorted, kin, vin, kout, vout, dt, tmp, st);
+  if (sorted || rc != NSORT_OK) return rc;
+  rc = ensure_pairs_smem_attr<V>();
   if (rc != NSORT_OK) return rc;
   char *t = static_cast<char *>(tmp);
   uint32_t *kb[2] = {kout, p.merge_passes ? reinterpret_cast<uint32_t *>(t + p.keys_off) : nullptr};

@@ -43,16 +43,16 @@ int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void 
 int sort_pairs_impl(const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout,
                     int64_t n, int dt, void *tmp, cudaStream_t st);
 
-// Digit sorts (radix.cu), for plans whose scratch holds one (radix_fits).
-bool radix_fits(const Plan &p, bool pairs, int key_bytes);
-int radix_sort_keys(const Plan &p, const uint32_t *in, uint32_t *out, int dt, void *tmp,
-                    cudaStream_t st);
-int radix_sort_keys64(const Plan &p, const uint64_t *in, uint64_t *out, int dt, void *tmp,
-                      cudaStream_t st);
-int radix_sort_pairs(const Plan &p, const uint32_t *in, const uint32_t *vin, uint32_t *out,
-                     uint32_t *vout, int dt, void *tmp, cudaStream_t st);
-int radix_sort_pairs64(const Plan &p, const uint32_t *in, const uint64_t *vin, uint32_t *out,
-                       uint64_t *vout, int dt, void *tmp, cudaStream_t st);
+// Digit sorts (radix.cu) of a plan; *sorted says whether there is one for it
+// (else nothing was done).
+int radix_sort_keys(const Plan &p, bool *sorted, const uint32_t *in, uint32_t *out, int dt,
+                    void *tmp, cudaStream_t st);
+int radix_sort_keys64(const Plan &p, bool *sorted, const uint64_t *in, uint64_t *out, int dt,
+                      void *tmp, cudaStream_t st);
+int radix_sort_pairs(const Plan &p, bool *sorted, const uint32_t *in, const uint32_t *vin,
+                     uint32_t *out, uint32_t *vout, int dt, void *tmp, cudaStream_t st);
+int radix_sort_pairs64(const Plan &p, bool *sorted, const uint32_t *in, const uint64_t *vin,
+                       uint32_t *out, uint64_t *vout, int dt, void *tmp, cudaStream_t st);
 
 size_t segmented_temp_bytes(int kind, uint64_t n, uint64_t nseg);
 
@@ -94,7 +94,8 @@ int merge_runs_impl(const void *kin, const uint32_t *vin, void *kout, uint32_t *
 enum TraceKernel {
   TK_TILE_SORT_KEYS = 0, TK_TILE_SORT_PAIRS, TK_PARTITION, TK_MERGE_KEYS, TK_MERGE_PAIRS,
   TK_SEG_BIN, TK_SEG_SORT, TK_SEG_MERGE, TK_SEG_COPY, TK_TILE_SORT_KEYS64, TK_MERGE_KEYS64,
-  TK_SAMPLE_MERGE, TK_MERGE4_BOUNDS, TK_MERGE4_KEYS, TK_RADIX_HIST, TK_RADIX_PASS
+  TK_SAMPLE_MERGE, TK_MERGE4_BOUNDS, TK_MERGE4_KEYS, TK_RADIX_HIST, TK_RADIX_PASS,
+  TK_RADIX_CLUSTER
 };
 
 // Brackets one kernel launch with CUDA events on its stream while tracing

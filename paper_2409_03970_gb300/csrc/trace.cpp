@@ -19,7 +19,7 @@ const char *const kKernelNames[] = {"tile_sort_keys", "tile_sort_pairs", "partit
                                     "segmented_sort", "segmented_merge", "segmented_copy",
                                     "tile_sort_keys64", "merge_keys64",
                                     "sample_merge",   "merge4_bounds",   "merge4_keys",
-                                    "radix_histogram", "radix_pass"};
+                                    "radix_histogram", "radix_pass",      "radix_cluster"};
 constexpr int kNumKernels = sizeof(kKernelNames) / sizeof(kKernelNames[0]);
 
 struct Rec {

@@ -1,9 +1,10 @@
-"""The digit passes of large plain sorts (csrc/radix.cu) against the oracle,
-bit for bit: sizes around a tile's edges (16384 keys or pairs, 8192 64-bit
-keys) on both sides of the smallest digit sort, distributions for each way of
-ranking (keys that agree in the sorted digits, keys that do not, a mix, one
-digit for a whole tile), keys equal to the padding of the last tile, in
-place, and buffers of any alignment.  Sorts are exact: no tolerance."""
+"""The digit sorts of arrays beyond one tile (csrc/radix.cu) against the
+oracle, bit for bit, at the sizes where the route changes (one cluster of 16
+CTAs, passes of tiles that all run at once, look-back passes) and at the edges
+of their tiles; distributions for each way of ranking (keys that agree in the
+sorted digits, keys that do not, a mix, one digit for a whole tile), keys
+equal to the padding of the last tile, in place, and buffers of any
+alignment.  Sorts are exact: no tolerance."""
 import numpy as np
 import pytest
 
@@ -70,65 +71,64 @@ def run(ns, kind, dt, keys, vals, inplace=False, offset=0):
     trace = ns.nsort_trace_read()
     ns.nsort_trace_enable(False)
     assert bool((tmp[need:] == 0x5A).all()), "wrote past the scratch"
-    passes = trace.get("radix_pass", {"launches": 0})["launches"]
+    route = sorted(k for k in trace if k.startswith("radix") or k.startswith("merge"))
+    if "radix_pass" in trace:
+        assert trace["radix_pass"]["launches"] == keys.dtype.itemsize
     out = [x.cpu().numpy().view(keys.dtype if i == 0 else vals.dtype)
            for i, x in enumerate([ko] + ([] if vo is None else [vo]))]
-    return passes, out
+    return route, out
 
 
-def smallest(ns, kind, dt):
-    """The smallest size that is sorted by digits (by bisection on the trace)."""
-    lo, hi = 8193, 1 << 23
-    wide = dt in inputs.KEY64_DTYPES
-    while lo < hi:
-        mid = (lo + hi) // 2
-        k = np.zeros(mid, np.uint64 if wide else np.uint32)
-        v = None if kind == ns.KIND_KEYS else np.zeros(mid, np.uint64 if kind == ns.KIND_PAIRS64
-                                                       else np.uint32)
-        passes, _ = run(ns, kind, dt, k, v)
-        if passes:
-            hi = mid
-        else:
-            lo = mid + 1
-    return lo
-
-
+CLUSTER, PASSES = ["radix_cluster"], ["radix_histogram", "radix_pass"]
 DISTS = ["uniform", "sorted", "dup16", "zipf", "low", "ones"]
+
+
+def sizes32(merge_tile):
+    """(n, route) of 32-bit keys and pairs: one cluster from two sort tiles
+    on, passes while 2 CTAs per SM hold all tiles, then look-back passes."""
+    at_once = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    clusters = (at_once // 4) * 4 * 4096
+    return [(merge_tile + 1, CLUSTER), (32768, CLUSTER), (32769, CLUSTER), (65536, CLUSTER),
+            (65537, None), (131072, None), (131073, None), (200_003, PASSES),
+            (clusters, PASSES), (clusters + 1, PASSES), (at_once * 10240 + 1, PASSES),
+            (at_once * 16384 + 1, PASSES)]
+
+
+def sizes64():
+    at_once = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    return [((5 << 18) - 1, ["merge_keys64"]), (5 << 18, PASSES), (at_once * 6144 + 1, PASSES),
+            (at_once * 8192, PASSES), (at_once * 8192 + 1, PASSES), ((1 << 22) - 1, PASSES)]
 
 
 @pytest.mark.parametrize("dt", ["u32", "i32", "f32", "i64", "f64"])
 def test_keys(ns, dt):
     wide = dt in inputs.KEY64_DTYPES
-    tile = 8192 if wide else 16384
-    first = smallest(ns, ns.KIND_KEYS, dt)
-    sizes = [first - 1, first, -(-first // tile) * tile, -(-first // tile) * tile + 1,
-             (1 << 22) + 3 * tile - 1]
-    for i, n in enumerate(sizes):
+    for i, (n, want_route) in enumerate(sizes64() if wide else sizes32(16384)):
         for dist in DISTS:
-            if wide and dist == "zipf":
+            if wide and dist == "zipf" or (n > 3_000_000 and dist in ("sorted", "low")):
                 continue
             x = draw(n, dt, dist, seed=n)
             want = oracle.sort_keys64(x, dt) if wide else oracle.sort_keys(x, dt)
-            passes, (got,) = run(ns, ns.KIND_KEYS, dt, x, None, inplace=i % 2 == 1, offset=i % 3)
-            assert passes == (0 if i == 0 else x.itemsize)
+            route, (got,) = run(ns, ns.KIND_KEYS, dt, x, None, inplace=i % 2 == 1, offset=i % 3)
+            assert want_route is None or route == want_route
             np.testing.assert_array_equal(got, want, err_msg=f"{n} {dist}")
 
 
 @pytest.mark.parametrize("vbytes", [4, 8])
 def test_pairs(ns, vbytes):
     kind = ns.KIND_PAIRS if vbytes == 4 else ns.KIND_PAIRS64
-    first = smallest(ns, kind, "f32")
-    sizes = [first - 1, first, -(-first // 16384) * 16384, -(-first // 16384) * 16384 + 1]
-    for i, n in enumerate(sizes):
+    for i, (n, want_route) in enumerate(sizes32(8192)):
         # (pairs64 takes 16-byte aligned outputs only)
         offset = (i % 3) if vbytes == 4 else 0
         for dist in DISTS:
+            if n > 3_000_000 and dist in ("sorted", "low"):
+                continue
             dt = ["f32", "i32", "u32"][i % 3]
             x = draw(n, dt, dist, seed=n)
             order = np.arange(n, dtype=np.uint32)
             wk, perm = oracle.sort_pairs(x, order, dt)
             v = order if vbytes == 4 else inputs.counter_u64(n, 7, 0, n)
-            passes, (gk, gv) = run(ns, kind, dt, x, v, inplace=i % 2 == 1, offset=offset)
-            assert passes == (0 if i == 0 else 4)
+            route, (gk, gv) = run(ns, kind, dt, x, v, inplace=i % 2 == 1, offset=offset)
+            assert want_route is None or route == want_route
             np.testing.assert_array_equal(gk, wk, err_msg=f"{n} {dist}")
             np.testing.assert_array_equal(gv, v[perm], err_msg=f"{n} {dist}")
