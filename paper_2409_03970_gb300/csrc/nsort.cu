@@ -469,6 +469,8 @@ struct DescTiles {
   static constexpr bool kAnyStart = true;    // segments start anywhere
   const PairTile *desc;
   const unsigned long long *count;
+  const int *max_level;   // the batch's deepest level; this one is level k
+  int k;
   K *buf0, *buf1;
   uint32_t *vbuf0, *vbuf1;
   int dt;
@@ -664,6 +666,9 @@ __global__ void __launch_bounds__(NT, PAIRS ? 3 : 4) merge_tma_kernel(
     const K *__restrict__ src, const V *__restrict__ vsrc, K *__restrict__ dst,
     V *__restrict__ vdst, int64_t n, const GEOM geom, int64_t num_tiles_arg,
     const int64_t *__restrict__ split, int *status, K *samp, int reverse) {
+  if constexpr (GEOM::kDesc) {   // (an empty level: see seg_level_wait)
+    if (*(const volatile int *)geom.max_level < geom.k) pdl_trigger();
+  }
   pdl_wait();      // the previous kernel of the stream has finished writing
   int64_t num_tiles = num_tiles_arg;
   if constexpr (GEOM::kDesc) num_tiles = (int64_t)*geom.count;
@@ -2276,13 +2281,23 @@ __device__ __forceinline__ int ceil_log2_i64(int64_t x) {
   return p;
 }
 
+// Start of a kernel of level k: waits for the kernel before it.  If no
+// segment has k levels (max_level is final before the first level's kernels
+// are launched), neither this kernel nor any later one of the batch has
+// anything to do, and the next may start to wait at once: an empty level's
+// three kernels then cost little more than their turns.
+__device__ __forceinline__ void seg_level_wait(const int *max_level, int k) {
+  if (*(const volatile int *)max_level < k) pdl_trigger();
+  pdl_wait();      // the previous kernel of the stream has finished writing
+}
+
 // Grid-stride over the segments; nothing to do (and an immediate return)
 // when the offsets were malformed or no segment has k levels.
 __global__ void seg_describe_kernel(const int64_t *__restrict__ off, int64_t nseg,
                                     int64_t min_len, int tile, int k, int mt,
                                     const int *status, const int *max_level,
                                     unsigned long long *count, int64_t *__restrict__ tile_seg) {
-  pdl_wait();      // the previous kernel of the stream has finished writing
+  seg_level_wait(max_level, k);
   if (*status != NSORT_OK || *max_level < k) return;
   const int64_t run = (int64_t)tile << (k - 1);
   const int64_t tpp = (2 * run + mt - 1) / mt;
@@ -2318,8 +2333,29 @@ __device__ __forceinline__ void seg_partition_tile(const int64_t *__restrict__ o
   const int in1 = (P - (k - 1)) & 1;   // level k-1 of this segment is in buf1
   const K *A = (in1 ? buf1 : buf0) + o + pair0;
   const K *B = A + la;
-  int64_t a0 = merge_path_global(A, la, B, lb, d0);
-  int64_t a1 = d1 == la + lb ? la : merge_path_global(A, la, B, lb, d1);
+  // both co-ranks at once: their loads are in flight together
+  int64_t a0 = d0 - lb > 0 ? d0 - lb : 0, h0 = d0 < la ? d0 : la;
+  int64_t a1 = d1 - lb > 0 ? d1 - lb : 0, h1 = d1 < la ? d1 : la;
+  while (a0 < h0 || a1 < h1) {
+    const int64_t m0 = (a0 + h0) >> 1, m1 = (a1 + h1) >> 1;
+    K x0 = 0, y0 = 0, x1 = 0, y1 = 0;
+    if (a0 < h0) {
+      x0 = __ldg(A + m0);
+      y0 = __ldg(B + (d0 - 1 - m0));
+    }
+    if (a1 < h1) {
+      x1 = __ldg(A + m1);
+      y1 = __ldg(B + (d1 - 1 - m1));
+    }
+    if (a0 < h0) {
+      if (x0 <= y0) a0 = m0 + 1;
+      else h0 = m0;
+    }
+    if (a1 < h1) {
+      if (x1 <= y1) a1 = m1 + 1;
+      else h1 = m1;
+    }
+  }
   clamp_coranks(la, lb, d0, d1, a0, a1);
   PairTile g;
   g.out0 = o + pair0 + d0;
@@ -2334,10 +2370,10 @@ __device__ __forceinline__ void seg_partition_tile(const int64_t *__restrict__ o
 
 template <typename K>
 __global__ void seg_partition_kernel(const int64_t *__restrict__ off, int tile, int k, int mt,
-                                     const unsigned long long *count,
+                                     const int *max_level, const unsigned long long *count,
                                      const int64_t *__restrict__ tile_seg,
                                      const K *buf0, const K *buf1, PairTile *__restrict__ desc) {
-  pdl_wait();      // the previous kernel of the stream has finished writing
+  seg_level_wait(max_level, k);
   const int64_t ntiles = (int64_t)*count;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ntiles;
        t += (int64_t)gridDim.x * blockDim.x)
@@ -2357,6 +2393,8 @@ static void launch_seg_level_merge(const SegLevelArgs &a, cudaStream_t st) {
   DescTiles<K> geom;
   geom.desc = static_cast<const PairTile *>(a.desc);
   geom.count = a.count;
+  geom.max_level = a.max_level;
+  geom.k = a.k;
   geom.buf0 = a.kout;
   geom.buf1 = a.ktmp;
   geom.vbuf0 = a.vout;
@@ -2383,7 +2421,7 @@ int launch_segmented_level(const SegLevelArgs &a, cudaStream_t st) {
     TraceScope tr(TK_PARTITION, st);
     const int64_t blocks = (a.max_tiles + 255) / 256;
     launch_pdl(seg_partition_kernel<uint32_t>, (unsigned)(blocks < 1024 ? blocks : 1024), 256, 0, st,
-               a.off, a.tile, a.k, mt, (const unsigned long long *)a.count,
+               a.off, a.tile, a.k, mt, a.max_level, (const unsigned long long *)a.count,
                (const int64_t *)a.tile_seg, (const uint32_t *)a.kout, (const uint32_t *)a.ktmp,
                static_cast<PairTile *>(a.desc));
   }

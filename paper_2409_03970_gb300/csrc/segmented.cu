@@ -5,8 +5,9 @@
 //                            the W_t-input network (W_t = 8 or 16);
 //   small  L <= 32 * IPT     one warp: column sort of IPT keys per lane and
 //                            the warp flip merger (IPT = 8 or 16);
-//   medium L <= 16 NT        one CTA: tile sort with the active size rounded
-//                            up to a power of two;
+//   medium L <= 16 NT        keys: a group of 1, 2, 4 or 8 warps per segment
+//                            (at most 1024 keys a warp), as many groups as fit
+//                            a CTA; pairs: one CTA;
 //   large  L >  16 NT        tile sorts of the segment's TILE-key tiles
 //                            (level 0; keys take 32 per thread, TILE = 32 NT,
 //                            pairs 16, TILE = 16 NT), then one merge level per
@@ -33,6 +34,7 @@
 #include <type_traits>
 
 #include "nsort.h"
+#include "launch.h"
 #include "nsort_internal.h"
 #include "sort_device.cuh"
 #include "tma_device.cuh"
@@ -42,15 +44,16 @@ namespace seg {
 
 constexpr int MAXLV = 40;          // merge levels a segment can need (2^40 keys / 4096)
 constexpr int MIN_TILE = 256 * 16; // smallest tile over the configurations
+constexpr int CLASSES = 4;         // medium segments of at most 1024 << c keys (pairs: all in 0)
 
 struct Ctrl {
   int status;                          // NSORT_OK, NSORT_EINVAL (offsets), NSORT_ETIMEOUT
   int max_level;
   unsigned long long next_item;        // queue head
-  unsigned long long n_tiny, n_small, n_medium;
+  unsigned long long n_tiny, n_small, n_medium[CLASSES];
   unsigned long long bucket_tiles[MAXLV + 1];   // tiles of large segments needing b levels
   unsigned long long bucket_base[MAXLV + 2];    // exclusive prefix of bucket_tiles
-  unsigned long long q_medium, q_small, q_tiny, q_total;
+  unsigned long long q_medium[CLASSES], q_small, q_tiny, q_total;   // first items
   unsigned long long lvl_count[MAXLV + 2];      // merge tiles of level k (launch_segmented_level)
 };
 
@@ -65,11 +68,15 @@ struct Params {
   int64_t nseg;
   int64_t n;
   Ctrl *ctrl;
+  // Every segment is in one list only, so each array of nseg entries holds
+  // two lists, one from either end: tiny and medium class 0, small and
+  // medium class 1, medium classes 2 and 3.
   int *tiny_list;
   int *small_list;
   int *medium_list;
   int64_t *slot_base;    // large segment -> first slot of its tiles
   int *owner;            // slot -> large segment
+  uint32_t arith, flip;  // the key map of the type: b ^ ((b >> 31 & arith) | flip)
   int dt;
   int tile;              // keys per level-0 tile: NT * 32 (keys) or NT * 16 (pairs)
   int mt;                // longest medium segment: NT * 16
@@ -82,6 +89,22 @@ __device__ __forceinline__ int ceil_log2(int64_t x) {
   int p = 0;
   while ((int64_t(1) << p) < x) ++p;
   return p;
+}
+
+// to_key and from_key of the batch's type.
+__device__ __forceinline__ uint32_t map_in(const Params &p, uint32_t b) {
+  return b ^ (((uint32_t)((int32_t)b >> 31) & p.arith) | p.flip);
+}
+__device__ __forceinline__ uint32_t map_out(const Params &p, uint32_t k) {
+  return k ^ (((uint32_t)((int32_t)~k >> 31) & p.arith) | p.flip);
+}
+
+// Entry i of medium class c's list.
+__device__ __forceinline__ int *medium_entry(const Params &p, int c, unsigned long long i) {
+  if (c == 0) return p.tiny_list + (p.nseg - 1 - (int64_t)i);
+  if (c == 1) return p.small_list + (p.nseg - 1 - (int64_t)i);
+  if (c == 2) return p.medium_list + i;
+  return p.medium_list + (p.nseg - 1 - (int64_t)i);
 }
 
 // ---- set-up kernels ----------------------------------------------------------
@@ -104,49 +127,76 @@ __global__ void seg_classify_kernel(Params p) {
   } else if (L <= 32 * p.small_ipt) {
     p.small_list[atomicAdd(&c->n_small, 1ull)] = (int)s;
   } else if (L <= p.mt) {
-    p.medium_list[atomicAdd(&c->n_medium, 1ull)] = (int)s;
+    int k = 0;
+    if (!p.vin)
+      while ((1024 << k) < L) ++k;   // (L <= 8192)
+    *medium_entry(p, k, atomicAdd(&c->n_medium[k], 1ull)) = (int)s;
   } else {
     const int64_t T = (L + p.tile - 1) / p.tile;
     p.slot_base[s] = (int64_t)atomicAdd(&c->bucket_tiles[ceil_log2(T)], (unsigned long long)T);
   }
 }
 
-// Lays out the work queue (one thread).
+// Lays out the work queue (one warp).
 __global__ void seg_plan_kernel(Params p) {
+  pdl_wait();      // the previous kernel of the stream has finished writing
   Ctrl *c = p.ctrl;
+  const int lane = threadIdx.x;
   if (c->status != NSORT_OK) {
-    c->q_total = 0;
+    if (lane == 0) c->q_total = 0;
     return;
   }
-  unsigned long long base = 0;
-  int maxlv = 0;
-  for (int b = 0; b <= MAXLV; ++b) {
-    c->bucket_base[b] = base;
-    base += c->bucket_tiles[b];
-    if (c->bucket_tiles[b]) maxlv = b;
+  // exclusive prefix of the buckets' tiles, lanes taking buckets l and 32 + l
+  const unsigned long long t0 = c->bucket_tiles[lane];
+  const unsigned long long t1 = 32 + lane <= MAXLV ? c->bucket_tiles[32 + lane] : 0;
+  unsigned long long s0 = t0, s1 = t1;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long x0 = __shfl_up_sync(0xffffffffu, s0, o);
+    const unsigned long long x1 = __shfl_up_sync(0xffffffffu, s1, o);
+    if (lane >= o) {
+      s0 += x0;
+      s1 += x1;
+    }
   }
-  c->bucket_base[MAXLV + 1] = base;
-  c->q_medium = base;
-  c->q_small = c->q_medium + c->n_medium;
+  s1 += __shfl_sync(0xffffffffu, s0, 31);
+  c->bucket_base[lane] = s0 - t0;
+  if (32 + lane <= MAXLV + 1) c->bucket_base[32 + lane] = s1 - t1;
+  const unsigned m0 = __ballot_sync(0xffffffffu, t0 != 0), m1 = __ballot_sync(0xffffffffu, t1 != 0);
+  unsigned long long base = __shfl_sync(0xffffffffu, s1, 31);
+  if (lane) return;
   const unsigned long long warps = p.nt / 32;
+  for (int k = CLASSES - 1; k >= 0; --k) {   // the longest first
+    c->q_medium[k] = base;
+    const unsigned long long per = p.vin ? 1 : warps >> k;   // segments an item
+    base += (c->n_medium[k] + per - 1) / per;
+  }
+  c->q_small = base;
   c->q_tiny = c->q_small + (c->n_small + warps - 1) / warps;
   c->q_total = c->q_tiny + (c->n_tiny + p.nt - 1) / p.nt;
-  c->max_level = maxlv;
+  c->max_level = m1 ? 63 - __clz(m1) : (m0 ? 31 - __clz(m0) : 0);
 }
 
-// One warp per segment: gives each large segment its global slot range and
-// records the owner of every slot.
+// Gives each large segment its global slot range and records the owner of
+// every slot: a lane per segment, the warp together for each large one.
 __global__ void seg_owner_kernel(Params p) {
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  pdl_wait();      // the previous kernel of the stream has finished writing
+  const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
-  if (w >= p.nseg || p.ctrl->status != NSORT_OK) return;
-  const int64_t L = p.off[w + 1] - p.off[w];
-  if (L <= p.mt) return;
-  const int64_t T = (L + p.tile - 1) / p.tile;
-  const int64_t g = (int64_t)p.ctrl->bucket_base[ceil_log2(T)] + p.slot_base[w];
-  __syncwarp();
-  if (lane == 0) p.slot_base[w] = g;
-  for (int64_t i = lane; i < T; i += 32) p.owner[g + i] = (int)w;
+  if (p.ctrl->status != NSORT_OK) return;
+  const int64_t L = w < p.nseg ? p.off[w + 1] - p.off[w] : 0;
+  const bool large = L > p.mt;
+  int64_t T = 0, g = 0;
+  if (large) {
+    T = (L + p.tile - 1) / p.tile;
+    g = (int64_t)p.ctrl->bucket_base[ceil_log2(T)] + p.slot_base[w];
+    p.slot_base[w] = g;
+  }
+  for (unsigned m = __ballot_sync(0xffffffffu, large); m; m &= m - 1) {
+    const int l = __ffs(m) - 1;
+    const int64_t Tl = __shfl_sync(0xffffffffu, T, l), gl = __shfl_sync(0xffffffffu, g, l);
+    for (int64_t i = lane; i < Tl; i += 32) p.owner[gl + i] = (int)(w - lane + l);
+  }
 }
 
 // ---- the persistent kernel ------------------------------------------------
@@ -168,9 +218,10 @@ __device__ __forceinline__ int elem_pos(K e) {
   return (int)((uint64_t)e & 0xFFFFu);
 }
 
-// Tile sort with an active size m (a power of two, 512 <= m <= NT*16): only
+// Tile sort with an active size m (a multiple of 512, up to NT*16): only
 // the first m/16 threads hold data; all threads take part in the barriers.
-// On return thread t (< m/16) holds sorted elements [16t, 16t + 16).
+// On return thread t (< m/16) holds sorted elements [16t, 16t + 16).  The
+// last run of a level may be short or have no partner (it stays as it is).
 template <int NT, typename K>
 __device__ __forceinline__ void sort_tile_dyn(K (&r)[16], K *s, int m) {
   const int tid = threadIdx.x;
@@ -189,11 +240,12 @@ __device__ __forceinline__ void sort_tile_dyn(K (&r)[16], K *s, int m) {
 #pragma unroll 1
   for (int run = 512; run < m; run <<= 1) {
     __syncthreads();
-    if (e0 < m) {
-      const int g0 = e0 & ~(2 * run - 1);
+    const int g0 = e0 & ~(2 * run - 1);
+    const int nb = m - g0 - run < run ? m - g0 - run : run;   // of the pair's second run
+    if (e0 < m && nb > 0) {
       const int diag = e0 - g0;
-      const int ai = merge_path_smem(s, g0, run, g0 + run, run, diag);
-      serial_merge<16, false>(s, g0 + ai, g0 + run, g0 + run + diag - ai, g0 + 2 * run, r, unused);
+      const int ai = merge_path_smem(s, g0, run, g0 + run, nb, diag);
+      serial_merge<16, false>(s, g0 + ai, g0 + run, g0 + run + diag - ai, g0 + run + nb, r, unused);
     }
     if (2 * run < m) {
       __syncthreads();
@@ -205,87 +257,141 @@ __device__ __forceinline__ void sort_tile_dyn(K (&r)[16], K *s, int m) {
   }
 }
 
-// Sorts `count` elements of a segment starting at kin[base] with one CTA and
-// active size m; stores them (mapped back when `final_map`) at kdst[base].
-template <int NT, bool PAIRS>
-__device__ void block_sort_range(const Params &p, void *smem, int64_t base, int count, int m,
-                                 uint32_t *kdst, uint32_t *vdst, bool final_map) {
-  using K = typename std::conditional<PAIRS, uint64_t, uint32_t>::type;
-  K *s = static_cast<K *>(smem);
-  const int tid = threadIdx.x;
-  const int e0 = tid * 16;
-  K r[16];
-  if (e0 < m) {
-    const int act = m / 16;     // active threads; loads are striped over them
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int e = tid + act * j;
-      r[j] = e < count ? make_elem<K>(to_key(p.kin[base + e], p.dt), e) : (K)~(K)0;
-    }
-  }
-  sort_tile_dyn<NT>(r, s, m);
-  uint32_t vo[16];
-  if (PAIRS && e0 < m) {
-#pragma unroll
-    for (int k = 0; k < 16; ++k) vo[k] = e0 + k < count ? p.vin[base + elem_pos(r[k])] : 0u;
-  }
-  const int dto = final_map ? p.dt : (int)DT_U32;
-  // thread t holds sorted elements [16t, 16t + 16): staged in shared memory
-  // (padded; keys, then values for pairs) so that the global stores are
-  // coalesced whatever the segment's alignment
-  uint32_t *sk = reinterpret_cast<uint32_t *>(smem);
-  uint32_t *sv = sk + padded_len<uint32_t>(m);
-  __syncthreads();   // s is no longer read; every value gathered (vdst may alias vin)
-  if (e0 < m) {
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      if (e0 + k < count) {
-        sk[pidx<uint32_t>(e0 + k)] = from_key(elem_key(r[k]), dto);
-        if (PAIRS) sv[pidx<uint32_t>(e0 + k)] = vo[k];
-      }
-    }
-  }
-  __syncthreads();
-  for (int e = tid; e < count; e += NT) {
-    kdst[base + e] = sk[pidx<uint32_t>(e)];
-    if (PAIRS) vdst[base + e] = sv[pidx<uint32_t>(e)];
-  }
-}
-
 struct Best32Columns {
   template <typename K>
   __device__ __forceinline__ static void sort(K (&r)[32]) { column_sort_net<NET_BEST, 32>(r); }
 };
 
-// Level-0 tile of a large keys-only segment: `count` keys at kin[base],
-// sorted with 32 keys per thread by the keys tile sort's code (the best
-// 32-input network, the warp merge, gapped block merges); stored (mapped
-// back when `final_map`) at kdst[base].
-template <int NT>
-__device__ void tile_sort32_range(const Params &p, void *smem, int64_t base, int count,
-                                  uint32_t *kdst, bool final_map) {
-  uint32_t *s = static_cast<uint32_t *>(smem);
-  const int tid = threadIdx.x;
+// What a group of warps sorts: kept in shared memory while it does, since the
+// 32 keys a thread holds leave no registers for it.
+struct GroupJob {
+  const uint32_t *in;
+  uint32_t *out;
+  const uint32_t *vin;   // pairs: the payloads
+  uint32_t *vout;
+  int count;      // 1 .. 1024 per warp of the group (pairs: 512)
+  int map;        // whether the keys are mapped back
+};
+
+// Sorts job[g], as group g of W warps of the CTA (sort_group32).  Every
+// thread of the group calls it, after thread 0 of the group wrote the job.
+// Bound by the integer ALU pipe like the plain tile sort.  A segment costs
+// as many warps as it fills (whole 16384-key tiles and power-of-two blocks
+// sorted 1.2 keys of padding per 4 of log-uniform lengths), and segments of
+// less than a CTA's keys share one: 5.9e8 keys in 100,000 segments up to
+// 65536 long take 4.32 ms here, 5.54 before, 3.8 at the rate of the plain
+// tile sort; 30,000 segments up to 20,000 long 557 us in all, 790 before.
+template <int W>
+__device__ __forceinline__ void group_sort(const Params &p, void *smem, GroupJob *job, int g) {
+  uint32_t *s = static_cast<uint32_t *>(smem) + g * (W * GROUP_WARP_WORDS);
+  const int tid = threadIdx.x & (32 * W - 1);
+  auto bar = [&] {
+    if constexpr (W == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(32 * W) : "memory");
+  };
+  volatile GroupJob *j = job + g;
+  bar();
+  const int c0 = (tid >> 5) * 1024 + (tid & 31);   // a warp loads and stores 1024 keys in a row
   uint32_t r[32];
+  int aw;   // warps that hold keys
+  {
+    const int left = j->count - c0;
+    const uint32_t *in = j->in + c0;
+    aw = (j->count + 1023) >> 10;
 #pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    const int e = tid + NT * j;
-    r[j] = e < count ? to_key(p.kin[base + e], p.dt) : 0xFFFFFFFFu;
+    for (int k = 0; k < 32; ++k) r[k] = 32 * k < left ? map_in(p, in[32 * k]) : 0xFFFFFFFFu;
   }
-  sort_tile_in_block<NT, 32, Best32Columns, uint32_t, true>(r, s);
-  const int dto = final_map ? p.dt : (int)DT_U32;
-  // thread t holds tile elements [32t, 32t + 32): staged in shared memory
-  // (padded, conflict-free both ways) so that the global stores are
-  // coalesced whatever the segment's alignment
-  const int e0 = tid * 32;
-  __syncthreads();   // every thread is done reading s in the last merge level
+  sort_group32<W, Best32Columns>(r, s, tid, aw, bar);
+  // thread t holds keys [32t, 32t + 32): staged in shared memory (padded,
+  // conflict-free both ways) so that the global stores are coalesced
+  // whatever the segment's alignment
+  bar();   // every thread is done reading s in the last merge level
+  if ((tid >> 5) < aw) {
+    const int pb = pidx<uint32_t>(tid * 32);
+    const uint32_t arith = j->map ? p.arith : 0u, flip = j->map ? p.flip : 0u;
 #pragma unroll
-  for (int k = 0; k < 32; ++k) s[pidx<uint32_t>(e0 + k)] = r[k];
+    for (int k = 0; k < 32; ++k)
+      s[pb + k] = r[k] ^ (((uint32_t)((int32_t)~r[k] >> 31) & arith) | flip);
+  }
+  bar();
+  const int left = j->count - c0;
+  uint32_t *out = j->out + c0;
+  const uint32_t *from = s + pidx<uint32_t>(c0);
+#pragma unroll
+  for (int k = 0; k < 32; ++k)
+    if (32 * k < left) out[32 * k] = from[33 * k];
+}
+
+// Sorts job[0], pairs, by the whole CTA: composites of key and position, 16 a
+// thread, by as many warps as hold pairs; the payloads wait in shared memory
+// and are taken by position.
+template <int NT>
+__device__ __forceinline__ void pairs_sort(const Params &p, void *smem, volatile GroupJob *j) {
+  uint64_t *s = static_cast<uint64_t *>(smem);
+  uint32_t *sv = reinterpret_cast<uint32_t *>(s + merge_smem_len<uint64_t>(NT * 16, 16));
+  const int tid = threadIdx.x;
+  const int c0 = (tid >> 5) * 512 + (tid & 31);   // a warp loads and stores 512 pairs in a row
+  __syncthreads();   // the job is there
+  uint64_t r[16];
+  int m;   // pairs sorted: whole warps
+  {
+    const int left = j->count - c0;
+    const uint32_t *in = j->in + c0, *vin = j->vin + c0;
+    uint32_t *to = sv + pidx<uint32_t>(c0);
+    m = (j->count + 511) & ~511;
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      r[k] = 32 * k < left ? make_elem<uint64_t>(map_in(p, in[32 * k]), c0 + 32 * k) : ~0ull;
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      if (32 * k < left) to[33 * k] = vin[32 * k];
+  }
+  sort_tile_dyn<NT>(r, s, m);
+  // thread t holds pairs [16t, 16t + 16): staged (padded) so that the global
+  // stores are coalesced whatever the segment's alignment
+  __syncthreads();   // s is no longer read, the payloads are all there
+  uint32_t *sk = reinterpret_cast<uint32_t *>(s);
+  uint32_t *so = sk + padded_len<uint32_t>(NT * 16);
+  static_assert(2 * padded_len<uint32_t>(NT * 16) <= 2 * merge_smem_len<uint64_t>(NT * 16, 16),
+                "keys and payloads fit where the composites were");
+  if (tid * 16 < m) {
+    const uint32_t arith = j->map ? p.arith : 0u, flip = j->map ? p.flip : 0u;
+    const int pb = pidx<uint32_t>(tid * 16);   // one pad block holds all 16
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const uint32_t key = elem_key(r[k]);
+      sk[pb + k] = key ^ (((uint32_t)((int32_t)~key >> 31) & arith) | flip);
+      so[pb + k] = sv[pidx<uint32_t>(elem_pos(r[k]) & (NT * 16 - 1))];
+    }
+  }
   __syncthreads();
+  const int left = j->count - c0;
+  uint32_t *out = j->out + c0, *vout = j->vout + c0;
+  const int pf = pidx<uint32_t>(c0);
 #pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    const int e = tid + NT * j;
-    if (e < count) kdst[base + e] = from_key(s[pidx<uint32_t>(e)], dto);
+  for (int k = 0; k < 16; ++k) {
+    if (32 * k < left) {
+      out[32 * k] = sk[pf + 33 * k];
+      vout[32 * k] = so[pf + 33 * k];
+    }
+  }
+}
+
+// The medium segments of class C (at most 1024 << C keys) of one item: one
+// per group of 1 << C warps.
+template <int NT, int C>
+__device__ __forceinline__ void medium_item(const Params &p, void *smem, GroupJob *job,
+                                            unsigned long long item) {
+  constexpr int W = 1 << C;
+  const int g = threadIdx.x / (32 * W);
+  const unsigned long long idx = item * (NT / (32 * W)) + g;
+  if (idx < p.ctrl->n_medium[C]) {   // the same in all of the group
+    if (!(threadIdx.x & (32 * W - 1))) {
+      const int sid = *medium_entry(p, C, idx);
+      const int64_t off = p.off[sid];
+      job[g] = {p.kin + off, p.kout + off, nullptr, nullptr, (int)(p.off[sid + 1] - off), 1};
+    }
+    group_sort<W>(p, smem, job, g);
   }
 }
 
@@ -300,7 +406,7 @@ __device__ void warp_sort_segment(const Params &p, int64_t sid) {
 #pragma unroll
   for (int k = 0; k < IPT; ++k) {
     const int e = lane + 32 * k;
-    r[k] = e < L ? make_elem<K>(to_key(p.kin[off + e], p.dt), e) : (K)~(K)0;
+    r[k] = e < L ? make_elem<K>(map_in(p, p.kin[off + e]), e) : (K)~(K)0;
   }
   column_sort(r);
   warp_merge<IPT>(r, lane);
@@ -314,7 +420,7 @@ __device__ void warp_sort_segment(const Params &p, int64_t sid) {
 #pragma unroll
   for (int k = 0; k < IPT; ++k) {
     if (e0 + k < L) {
-      p.kout[off + e0 + k] = from_key(elem_key(r[k]), p.dt);
+      p.kout[off + e0 + k] = map_out(p, elem_key(r[k]));
       if (PAIRS) p.vout[off + e0 + k] = vo[k];
     }
   }
@@ -329,7 +435,7 @@ __device__ void thread_sort_segment(const Params &p, int64_t sid) {
   K r[W];
 #pragma unroll
   for (int k = 0; k < W; ++k)
-    r[k] = k < L ? make_elem<K>(to_key(p.kin[off + k], p.dt), k) : (K)~(K)0;
+    r[k] = k < L ? make_elem<K>(map_in(p, p.kin[off + k]), k) : (K)~(K)0;
   column_sort(r);
   uint32_t vo[W];
   if (PAIRS) {
@@ -339,57 +445,77 @@ __device__ void thread_sort_segment(const Params &p, int64_t sid) {
 #pragma unroll
   for (int k = 0; k < W; ++k) {
     if (k < L) {
-      p.kout[off + k] = from_key(elem_key(r[k]), p.dt);
+      p.kout[off + k] = map_out(p, elem_key(r[k]));
       if (PAIRS) p.vout[off + k] = vo[k];
     }
   }
 }
 
-template <int NT, bool PAIRS>
-__global__ void __launch_bounds__(NT, PAIRS ? 1 : 2) seg_sort_kernel(Params p) {
+// MINB: CTAs per SM that the registers are bounded for.  Two for keys and for
+// large batches of pairs (4.4e7 pairs in 30,000 segments: 1107 against 1261
+// us with one); one where the pairs fill no more than a tile per SM, when a
+// tile's own time counts (100 segments of up to 65536 pairs: 109 against 119).
+template <int NT, bool PAIRS, int MINB>
+__global__ void __launch_bounds__(NT, MINB) seg_sort_kernel(Params p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long item_sh;
   // The queue's bin boundaries live in shared memory and are read per item:
   // held in registers for the whole loop they would cost the tile sorts
   // (at 2 CTAs of 512 threads, 64 registers a thread) registers they need.
-  __shared__ unsigned long long q_sh[4];   // medium, small, tiny, total
+  __shared__ unsigned long long q_sh[CLASSES + 3];   // medium classes, small, tiny, total
+  __shared__ GroupJob job[PAIRS ? 1 : NT / 32];
+  pdl_wait();      // the previous kernel of the stream has finished writing
   const int tid = threadIdx.x;
   Ctrl *c = p.ctrl;
+  if (tid < CLASSES) q_sh[tid] = c->q_medium[tid];
   if (tid == 0) {
-    q_sh[0] = c->q_medium;
-    q_sh[1] = c->q_small;
-    q_sh[2] = c->q_tiny;
-    q_sh[3] = c->q_total;
+    q_sh[CLASSES] = c->q_small;
+    q_sh[CLASSES + 1] = c->q_tiny;
+    q_sh[CLASSES + 2] = c->q_total;
   }
+  // Few items: the first half of the grid takes them all, about one CTA per
+  // SM, rather than two on some SMs and none on others.
+  if (2 * blockIdx.x >= gridDim.x && 2 * c->q_total <= gridDim.x) return;
   for (;;) {
     if (tid == 0) item_sh = atomicAdd(&c->next_item, 1ull);
     __syncthreads();
     const unsigned long long item = item_sh;
-    const unsigned long long q_medium = q_sh[0], q_small = q_sh[1], q_tiny = q_sh[2],
-                             q_total = q_sh[3];
+    const unsigned long long q_small = q_sh[CLASSES], q_tiny = q_sh[CLASSES + 1],
+                             q_total = q_sh[CLASSES + 2];
     __syncthreads();
     if (item >= q_total) break;
-    if (item < q_medium) {
+    if (item < q_sh[CLASSES - 1]) {
       // level 0: tile sort of one tile of a large segment (the whole sort,
       // key map included, when the segment fits one tile)
-      const int sid = p.owner[item];
-      const int64_t t = (int64_t)item - p.slot_base[sid];
-      const int64_t off = p.off[sid];
-      const int64_t L = p.off[sid + 1] - off;
-      const int P = ceil_log2((L + p.tile - 1) / p.tile);
-      const int64_t b0 = t * p.tile;
-      const int count = (int)(L - b0 < p.tile ? L - b0 : p.tile);
-      uint32_t *kd = (P & 1) ? p.ktmp : p.kout;
-      uint32_t *vd = (P & 1) ? p.vtmp : p.vout;
-      if (PAIRS) block_sort_range<NT, PAIRS>(p, smem_raw, off + b0, count, NT * 16, kd, vd, P == 0);
-      else tile_sort32_range<NT>(p, smem_raw, off + b0, count, kd, P == 0);
+      if (tid == 0) {
+        const int sid = p.owner[item];
+        const int64_t t = (int64_t)item - p.slot_base[sid];
+        const int64_t off = p.off[sid];
+        const int64_t L = p.off[sid + 1] - off;
+        const int P = ceil_log2((L + p.tile - 1) / p.tile);
+        const int64_t b0 = t * p.tile, at = off + b0;
+        const bool tmp = P & 1;
+        job[0] = {p.kin + at, (tmp ? p.ktmp : p.kout) + at, PAIRS ? p.vin + at : nullptr,
+                  PAIRS ? (tmp ? p.vtmp : p.vout) + at : nullptr,
+                  (int)(L - b0 < p.tile ? L - b0 : p.tile), P == 0};
+      }
+      if constexpr (PAIRS) pairs_sort<NT>(p, smem_raw, job);
+      else group_sort<NT / 32>(p, smem_raw, job, 0);
     } else if (item < q_small) {
-      const int sid = p.medium_list[item - q_medium];
-      const int64_t off = p.off[sid];
-      const int L = (int)(p.off[sid + 1] - off);
-      int m = 512;
-      while (m < L) m <<= 1;
-      block_sort_range<NT, PAIRS>(p, smem_raw, off, L, m, p.kout, p.vout, true);
+      if constexpr (PAIRS) {
+        if (tid == 0) {
+          const int sid = *medium_entry(p, 0, item - q_sh[0]);
+          const int64_t off = p.off[sid];
+          job[0] = {p.kin + off, p.kout + off, p.vin + off, p.vout + off,
+                    (int)(p.off[sid + 1] - off), 1};
+        }
+        pairs_sort<NT>(p, smem_raw, job);
+      } else {
+        if (NT == 512 && item < q_sh[2]) medium_item<512, 3>(p, smem_raw, job, item - q_sh[3]);
+        else if (item < q_sh[1]) medium_item<NT, 2>(p, smem_raw, job, item - q_sh[2]);
+        else if (item < q_sh[0]) medium_item<NT, 1>(p, smem_raw, job, item - q_sh[1]);
+        else medium_item<NT, 0>(p, smem_raw, job, item - q_sh[0]);
+      }
     } else if (item < q_tiny) {
       const unsigned long long idx = (item - q_small) * (NT / 32) + (tid >> 5);
       if (idx < c->n_small) {
@@ -445,21 +571,22 @@ nsort_seg_config g_cfg = {512, 16, 16, 0};
 
 template <int NT, bool PAIRS>
 size_t smem_bytes() {
-  using K = typename std::conditional<PAIRS, uint64_t, uint32_t>::type;
-  const size_t tile_b = sizeof(K) * merge_smem_len<K>(NT * 16, 16);
-  const size_t tile32_b = PAIRS ? 0 : sizeof(uint32_t) * block_smem_len<uint32_t>(NT, 32);
-  return tile_b > tile32_b ? tile_b : tile32_b;
+  if (PAIRS)
+    return sizeof(uint64_t) * merge_smem_len<uint64_t>(NT * 16, 16) +
+           sizeof(uint32_t) * padded_len<uint32_t>(NT * 16);
+  return sizeof(uint32_t) * (NT / 32) * GROUP_WARP_WORDS;
 }
 
-template <int NT, bool PAIRS>
+template <int NT, bool PAIRS, int MINB>
 int launch_sort(const Params &p, int blocks_per_sm, cudaStream_t st) {
   const size_t smem = smem_bytes<NT, PAIRS>();
   int dev = 0, sms = 0, occ = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaFuncSetAttribute(seg_sort_kernel<NT, PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      cudaFuncSetAttribute(seg_sort_kernel<NT, PAIRS, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, seg_sort_kernel<NT, PAIRS>, NT, smem) !=
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, seg_sort_kernel<NT, PAIRS, MINB>, NT,
+                                                    smem) !=
           cudaSuccess) {
     set_last_error(std::string("nsort_segmented set-up: ") + cudaGetErrorString(cudaGetLastError()));
     return NSORT_ECUDA;
@@ -467,7 +594,7 @@ int launch_sort(const Params &p, int blocks_per_sm, cudaStream_t st) {
   if (occ < 1) occ = 1;
   const int per_sm = blocks_per_sm > 0 && blocks_per_sm < occ ? blocks_per_sm : occ;
   TraceScope tr(TK_SEG_SORT, st);
-  seg_sort_kernel<NT, PAIRS><<<sms * per_sm, NT, smem, st>>>(p);
+  launch_pdl(seg_sort_kernel<NT, PAIRS, MINB>, (unsigned)(sms * per_sm), NT, smem, st, p);
   return NSORT_OK;
 }
 
@@ -541,6 +668,8 @@ int segmented_impl(const void *d_keys_in, void *d_keys_out, const uint32_t *d_va
   p.medium_list = reinterpret_cast<int *>(t + l.medium);
   p.slot_base = reinterpret_cast<int64_t *>(t + l.slot);
   p.owner = reinterpret_cast<int *>(t + l.owner);
+  p.arith = dtype == NSORT_F32 ? ~0u : 0u;
+  p.flip = dtype == NSORT_U32 ? 0u : 0x80000000u;
   p.dt = dtype;
   p.nt = cfg.block_threads;
   p.mt = cfg.block_threads * 16;
@@ -556,14 +685,25 @@ int segmented_impl(const void *d_keys_in, void *d_keys_out, const uint32_t *d_va
   {
     TraceScope tr(TK_SEG_BIN, st);
     seg::seg_classify_kernel<<<cblocks, 256, 0, st>>>(p);
-    seg::seg_plan_kernel<<<1, 1, 0, st>>>(p);
-    seg::seg_owner_kernel<<<(unsigned)((nseg * 32 + 255) / 256), 256, 0, st>>>(p);
+    launch_pdl(seg::seg_plan_kernel, 1, 32, 0, st, p);
+    launch_pdl(seg::seg_owner_kernel, cblocks, 256, 0, st, p);
   }
   int rc;
-  if (p.nt == 512) rc = pairs ? seg::launch_sort<512, true>(p, cfg.blocks_per_sm, st)
-                              : seg::launch_sort<512, false>(p, cfg.blocks_per_sm, st);
-  else rc = pairs ? seg::launch_sort<256, true>(p, cfg.blocks_per_sm, st)
-                  : seg::launch_sort<256, false>(p, cfg.blocks_per_sm, st);
+  const int per_sm = cfg.blocks_per_sm;
+  int dev = 0, sms = 0;
+  if (pairs && (cudaGetDevice(&dev) != cudaSuccess ||
+                cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)) {
+    set_last_error(std::string("nsort_segmented set-up: ") + cudaGetErrorString(cudaGetLastError()));
+    return NSORT_ECUDA;
+  }
+  if (!pairs)
+    rc = p.nt == 512 ? seg::launch_sort<512, false, 2>(p, per_sm, st)
+                     : seg::launch_sort<256, false, 2>(p, per_sm, st);
+  else if (p.nt == 512)
+    rc = n <= (uint64_t)sms * p.tile ? seg::launch_sort<512, true, 1>(p, per_sm, st)
+                                     : seg::launch_sort<512, true, 2>(p, per_sm, st);
+  else
+    rc = seg::launch_sort<256, true, 2>(p, per_sm, st);
   if (rc != NSORT_OK) return rc;
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

@@ -661,4 +661,72 @@ __device__ __forceinline__ void sort_tile_in_block(K (&r)[IPT], K *s) {
   }
 }
 
+// ---- sort by a group of warps ----------------------------------------------
+// Words of shared memory per warp of a group sort: 1024 keys and the gap
+// behind them, padded, or the warp's transpose buffer.
+constexpr int GROUP_WARP_WORDS = 1124;
+static_assert(GROUP_WARP_WORDS >= 32 * 33 &&
+                  16 * GROUP_WARP_WORDS >= padded_len<uint32_t>(16 * (1024 + 64)),
+              "a group's runs, gaps and transposes fit");
+
+// sort_tile_in_block for 32-bit keys, by the first `aw` of a group of W warps
+// (32 keys a thread, tid = thread in the group): sorts the 1024 aw keys in
+// their registers, so that thread t < 32 aw ends with keys 32 t .. 32 t + 31.
+// Only the warps that hold keys take part in the work; all W meet at the
+// barriers (bar), and s is the group's W * GROUP_WARP_WORDS words.  The last
+// run of a level may be short or have no partner (its keys stay where they
+// are).
+template <int W, class COLS, class BAR>
+__device__ __forceinline__ void sort_group32(uint32_t (&r)[32], uint32_t *s, int tid, int aw,
+                                             BAR bar) {
+  constexpr int GAP = block_gap<uint32_t>(32);
+  const int lane = tid & 31;
+  const bool on = (tid >> 5) < aw;
+  if (on) {
+    COLS::sort(r);
+    uint32_t *t = s + (tid >> 5) * (32 * 33);
+    warp_merge_level<1>(r, lane);
+    warp_merge_level<2>(r, lane);
+    warp_merge_level_t<3>(r, lane, t);
+    warp_merge_level_t<4>(r, lane, t);
+    warp_merge_level_t<5>(r, lane, t);
+  }
+  if (W == 1 || aw == 1) return;
+  const int act = 1024 * aw;
+  const int e0 = tid * 32;
+  // this thread's keys into the gapped layout of runs of 2^lr, and the
+  // largest keys behind a run that ends with this warp's
+  auto stage = [&](int lr) {
+    const int pb = pidx<uint32_t>(e0 + (e0 >> lr) * GAP);   // one pad block holds all 32
+#pragma unroll
+    for (int k = 0; k < 32; ++k) s[pb + k] = r[k];
+    const int wend = e0 + (32 - lane) * 32;   // end of the warp's keys (same in every lane)
+    if (!(wend & ((1 << lr) - 1)) || wend == act) {
+      const int gap0 = wend + ((wend - 1) >> lr) * GAP;
+      for (int j = lane; j < GAP; j += 32) s[pidx<uint32_t>(gap0 + j)] = ~0u;
+    }
+  };
+  bar();   // every warp is done with its transpose buffer
+  if (on) stage(10);
+#pragma unroll 1
+  for (int lr = 10; (1 << lr) < act; ++lr) {
+    bar();
+    const int run = 1 << lr;
+    const int g0 = e0 & ~(2 * run - 1);
+    const int left = act - g0 - run;   // of the pair's second run
+    const int nb = left < run ? left : run;
+    if (on && nb > 0) {
+      const int diag = e0 - g0;
+      const int a0 = g0 + (g0 >> lr) * GAP;   // run 2p and its gap, then run 2p+1
+      const int b0 = a0 + run + GAP;
+      const int ai = merge_path_smem(s, a0, run, b0, nb, diag);
+      serial_merge_gapped<32>(s, a0 + ai, b0 + diag - ai, r);
+    }
+    if (2 * run < act) {
+      bar();
+      if (on) stage(lr + 1);
+    }
+  }
+}
+
 }  // namespace nsort
