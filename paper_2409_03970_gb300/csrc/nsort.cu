@@ -77,9 +77,8 @@ __device__ __forceinline__ bool aligned16(const void *p) {
 // Tile sort, keys only.  Tile b covers [b*TILE, min((b+1)*TILE, n)); a short
 // last tile is padded with the largest key, which sorts behind every real
 // key and is never stored.  DT is the key type (its order-preserving map is
-// applied on load); FINAL maps the keys back on store (the tile sort is the
-// whole sort when n fits one tile).  in may equal out: each CTA reads its
-// whole tile before its first barrier and writes it after its last.
+// applied on load).  in may equal out: each CTA reads its whole tile before
+// its first barrier and writes it after its last.
 // Every SAMPLE-th output key of a sort stage (tile sort or merge pass) is
 // also written to a sample array; the next pass's partition searches the
 // samples first (section "sampled partition" below).
@@ -93,7 +92,7 @@ struct BestColumns {
   __device__ __forceinline__ static void sort(K (&r)[W]) { column_sort_net<NET_BEST, W>(r); }
 };
 
-template <int NT, int IPT, int DT, bool FINAL>
+template <int NT, int IPT, int DT>
 __global__ void __launch_bounds__(NT) tile_sort_keys_kernel(const uint32_t *in, uint32_t *out,
                                                             int64_t n, uint32_t *samp) {
   constexpr int TILE = NT * IPT;
@@ -125,9 +124,9 @@ __global__ void __launch_bounds__(NT) tile_sort_keys_kernel(const uint32_t *in, 
     }
   }
   sort_tile_in_block<NT, IPT, BestColumns>(r, s);
-  store_run<IPT, FINAL ? DT : DT_U32>(r, out + base, count, full);
+  store_run<IPT, DT_U32>(r, out + base, count, full);
   static_assert(SAMPLE % IPT == 0, "a sample starts a thread's run");
-  if (!FINAL && samp && !(tid & (SAMPLE / IPT - 1)) && tid * IPT < count)
+  if (samp && !(tid & (SAMPLE / IPT - 1)) && tid * IPT < count)
     store_keep_in_l2(samp + (base + tid * IPT) / SAMPLE, r[0]);
 }
 
@@ -137,7 +136,7 @@ __global__ void __launch_bounds__(NT) tile_sort_keys_kernel(const uint32_t *in, 
 // staged in shared memory and gathered by position at the end; 64-bit ones
 // are gathered by position from global memory, all of them before the
 // first store (in == out is allowed).
-template <int NT, int DT, bool FINAL, typename V = uint32_t>
+template <int NT, int DT, typename V = uint32_t>
 __global__ void __launch_bounds__(NT, 2) tile_sort_pairs_kernel(const uint32_t *kin,
                                                              const V *vin, uint32_t *kout,
                                                              V *vout, int64_t n, uint32_t *samp) {
@@ -177,7 +176,7 @@ __global__ void __launch_bounds__(NT, 2) tile_sort_pairs_kernel(const uint32_t *
       ko[k] = (uint32_t)(r[k] >> 32);
       vo[k] = sv[pidx<uint32_t>((int)(r[k] & 0xFFFFu) & (TILE - 1))];
     }
-    store_run<16, FINAL ? DT : DT_U32>(ko, kout + base, count, full);
+    store_run<16, DT_U32>(ko, kout + base, count, full);
     store_run<16, DT_U32>(vo, vout + base, count, full);
   } else {
     // keys first (every key was read before the block merges' barriers),
@@ -188,21 +187,21 @@ __global__ void __launch_bounds__(NT, 2) tile_sort_pairs_kernel(const uint32_t *
       ko[k] = (uint32_t)(r[k] >> 32);
       pos[k] = (int)(r[k] & 0xFFFFu) & (TILE - 1);
     }
-    store_run<16, FINAL ? DT : DT_U32>(ko, kout + base, count, full);
+    store_run<16, DT_U32>(ko, kout + base, count, full);
     V vo[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) vo[k] = tid * 16 + k < count ? vin[base + pos[k]] : V(0);
     __syncthreads();
     store_run<16, DT_U32>(vo, vout + base, count, full);
   }
-  if (!FINAL && samp && !(tid & (SAMPLE / 16 - 1)) && tid * 16 < count)
+  if (samp && !(tid & (SAMPLE / 16 - 1)) && tid * 16 < count)
     store_keep_in_l2(samp + (base + tid * 16) / SAMPLE, ko[0]);
 }
 
 // Tile sort, 64-bit keys (u64 / i64 / f64): the keys tile sort on 64-bit
 // words, NT * 16 keys per tile, the same networks and merges.  Every
 // SAMPLE-th output key goes to the sample array as for 32-bit keys.
-template <int NT, int DT, bool FINAL>
+template <int NT, int DT>
 __global__ void __launch_bounds__(NT) tile_sort_keys64_kernel(const uint64_t *in, uint64_t *out,
                                                               int64_t n, uint64_t *samp) {
   constexpr int TILE = NT * 16;
@@ -232,8 +231,8 @@ __global__ void __launch_bounds__(NT) tile_sort_keys64_kernel(const uint64_t *in
     }
   }
   sort_tile_in_block<NT, 16, Green16Columns>(r, s);
-  store_run<16, FINAL ? DT : DT_U64>(r, out + base, count, full);
-  if (!FINAL && samp && !(tid & (SAMPLE / 16 - 1)) && tid * 16 < count)
+  store_run<16, DT_U64>(r, out + base, count, full);
+  if (samp && !(tid & (SAMPLE / 16 - 1)) && tid * 16 < count)
     store_keep_in_l2(samp + (base + tid * 16) / SAMPLE, r[0]);
 }
 
@@ -1583,58 +1582,31 @@ static int launch_status(const char *what) {
 
 // ---- template dispatch (key type and "last pass" are compile-time) -------
 
-template <int DT, bool FIN>
+template <int DT>
 static void keys_sort_smem_attr() {
-  cudaFuncSetAttribute(tile_sort_keys_kernel<KEYS_SORT_NT, KEYS_SORT_IPT, DT, FIN>,
+  cudaFuncSetAttribute(tile_sort_keys_kernel<KEYS_SORT_NT, KEYS_SORT_IPT, DT>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KEYS_SORT_SMEM);
 }
 
 static void launch_tile_sort_keys(const uint32_t *in, uint32_t *out, int64_t n, int dt,
-                                  bool final_pass, unsigned grid, uint32_t *samp, cudaStream_t st) {
+                                  unsigned grid, uint32_t *samp, cudaStream_t st) {
   static std::atomic<uint64_t> done_mask{0};
   int dev = 0;
   cudaGetDevice(&dev);
   const uint64_t bit = dev < 64 ? (uint64_t(1) << dev) : 0;
   if (!bit || !(done_mask.load() & bit)) {   // opt in to the dynamic shared memory, once per device
-    keys_sort_smem_attr<DT_U32, false>();
-    keys_sort_smem_attr<DT_U32, true>();
-    keys_sort_smem_attr<DT_I32, false>();
-    keys_sort_smem_attr<DT_I32, true>();
-    keys_sort_smem_attr<DT_F32, false>();
-    keys_sort_smem_attr<DT_F32, true>();
+    keys_sort_smem_attr<DT_U32>();
+    keys_sort_smem_attr<DT_I32>();
+    keys_sort_smem_attr<DT_F32>();
     done_mask.fetch_or(bit);
   }
-#define NSORT_TSK(DT, FIN)                                                        \
-  tile_sort_keys_kernel<KEYS_SORT_NT, KEYS_SORT_IPT, DT, FIN>                             \
-      <<<grid, KEYS_SORT_NT, KEYS_SORT_SMEM, st>>>(                                       \
-      in, out, n, samp)
-  if (dt == DT_U32) { if (final_pass) NSORT_TSK(DT_U32, true); else NSORT_TSK(DT_U32, false); }
-  else if (dt == DT_I32) { if (final_pass) NSORT_TSK(DT_I32, true); else NSORT_TSK(DT_I32, false); }
-  else { if (final_pass) NSORT_TSK(DT_F32, true); else NSORT_TSK(DT_F32, false); }
+#define NSORT_TSK(DT)                                                                    \
+  tile_sort_keys_kernel<KEYS_SORT_NT, KEYS_SORT_IPT, DT>                                  \
+      <<<grid, KEYS_SORT_NT, KEYS_SORT_SMEM, st>>>(in, out, n, samp)
+  if (dt == DT_U32) NSORT_TSK(DT_U32);
+  else if (dt == DT_I32) NSORT_TSK(DT_I32);
+  else NSORT_TSK(DT_F32);
 #undef NSORT_TSK
-}
-
-// A whole sort in one CTA of NT threads x 16 keys (a tile of 16 NT keys).
-template <int NT>
-static void small_sort_nt(const uint32_t *in, uint32_t *out, int64_t n, int dt, cudaStream_t st) {
-  constexpr size_t smem = sizeof(uint32_t) * block_smem_len<uint32_t>(NT, 16);
-  static_assert(smem <= 48 * 1024, "fits the default dynamic shared memory");
-  if (dt == DT_U32) tile_sort_keys_kernel<NT, 16, DT_U32, true><<<1, NT, smem, st>>>(in, out, n, nullptr);
-  else if (dt == DT_I32) tile_sort_keys_kernel<NT, 16, DT_I32, true><<<1, NT, smem, st>>>(in, out, n, nullptr);
-  else tile_sort_keys_kernel<NT, 16, DT_F32, true><<<1, NT, smem, st>>>(in, out, n, nullptr);
-}
-
-// A sort that fits one tile of a smaller configuration takes the smallest
-// of 512, 2048 and 8192 keys (32, 128 or 512 threads x 16 keys) that holds
-// n, so that a short array does not pay for a full 16384-key tile.  Returns
-// false when n needs the full tile.
-static bool launch_small_sort(const uint32_t *in, uint32_t *out, int64_t n, int dt,
-                              cudaStream_t st) {
-  if (n <= 512) small_sort_nt<32>(in, out, n, dt, st);
-  else if (n <= 2048) small_sort_nt<128>(in, out, n, dt, st);
-  else if (n <= 8192) small_sort_nt<512>(in, out, n, dt, st);
-  else return false;
-  return true;
 }
 
 static void launch_merge_keys(const uint32_t *src, uint32_t *dst, int64_t n, int64_t run,
@@ -1647,9 +1619,9 @@ static void launch_merge_keys(const uint32_t *src, uint32_t *dst, int64_t n, int
 #undef NSORT_MK
 }
 
-template <int DT, bool FIN, typename V>
+template <int DT, typename V>
 static cudaError_t pairs_smem_attr() {
-  return cudaFuncSetAttribute(tile_sort_pairs_kernel<PAIRS_SORT_NT, DT, FIN, V>,
+  return cudaFuncSetAttribute(tile_sort_pairs_kernel<PAIRS_SORT_NT, DT, V>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)pairs_sort_smem<V>());
 }
@@ -1661,12 +1633,9 @@ static int ensure_pairs_smem_attr() {
   static std::atomic<uint64_t> done_mask{0};
   const uint64_t bit = dev < 64 ? (uint64_t(1) << dev) : 0;
   if (bit && (done_mask.load() & bit)) return NSORT_OK;
-  cudaError_t e = pairs_smem_attr<DT_U32, false, V>();
-  if (e == cudaSuccess) e = pairs_smem_attr<DT_U32, true, V>();
-  if (e == cudaSuccess) e = pairs_smem_attr<DT_I32, false, V>();
-  if (e == cudaSuccess) e = pairs_smem_attr<DT_I32, true, V>();
-  if (e == cudaSuccess) e = pairs_smem_attr<DT_F32, false, V>();
-  if (e == cudaSuccess) e = pairs_smem_attr<DT_F32, true, V>();
+  cudaError_t e = pairs_smem_attr<DT_U32, V>();
+  if (e == cudaSuccess) e = pairs_smem_attr<DT_I32, V>();
+  if (e == cudaSuccess) e = pairs_smem_attr<DT_F32, V>();
   if (e != cudaSuccess) return launch_status("cudaFuncSetAttribute");
   done_mask.fetch_or(bit);
   return NSORT_OK;
@@ -1674,14 +1643,14 @@ static int ensure_pairs_smem_attr() {
 
 template <typename V>
 static void launch_tile_sort_pairs(const uint32_t *kin, const V *vin, uint32_t *kout, V *vout,
-                                   int64_t n, int dt, bool final_pass, unsigned grid,
-                                   uint32_t *samp, cudaStream_t st) {
-#define NSORT_TSP(DT, FIN)                                                                  \
-  tile_sort_pairs_kernel<PAIRS_SORT_NT, DT, FIN, V><<<grid, PAIRS_SORT_NT, pairs_sort_smem<V>(), \
-                                                      st>>>(kin, vin, kout, vout, n, samp)
-  if (dt == DT_U32) { if (final_pass) NSORT_TSP(DT_U32, true); else NSORT_TSP(DT_U32, false); }
-  else if (dt == DT_I32) { if (final_pass) NSORT_TSP(DT_I32, true); else NSORT_TSP(DT_I32, false); }
-  else { if (final_pass) NSORT_TSP(DT_F32, true); else NSORT_TSP(DT_F32, false); }
+                                   int64_t n, int dt, unsigned grid, uint32_t *samp,
+                                   cudaStream_t st) {
+#define NSORT_TSP(DT)                                                                       \
+  tile_sort_pairs_kernel<PAIRS_SORT_NT, DT, V><<<grid, PAIRS_SORT_NT, pairs_sort_smem<V>(), \
+                                                 st>>>(kin, vin, kout, vout, n, samp)
+  if (dt == DT_U32) NSORT_TSP(DT_U32);
+  else if (dt == DT_I32) NSORT_TSP(DT_I32);
+  else NSORT_TSP(DT_F32);
 #undef NSORT_TSP
 }
 
@@ -1876,15 +1845,14 @@ static void launch_merge4(const uint32_t *src, uint32_t *dst, int64_t n, int64_t
 // ---- 64-bit keys -------------------------------------------------------------
 
 static void launch_tile_sort_keys64(const uint64_t *in, uint64_t *out, int64_t n, int dt,
-                                    bool final_pass, unsigned grid, uint64_t *samp,
-                                    cudaStream_t st) {
+                                    unsigned grid, uint64_t *samp, cudaStream_t st) {
   static_assert(KEYS64_SORT_SMEM <= 48 * 1024, "fits the default dynamic shared memory");
-#define NSORT_TSK64(DT, FIN)                                                            \
-  tile_sort_keys64_kernel<KEYS64_SORT_NT, DT, FIN><<<grid, KEYS64_SORT_NT, KEYS64_SORT_SMEM, \
-                                                     st>>>(in, out, n, samp)
-  if (dt == DT_U64) { if (final_pass) NSORT_TSK64(DT_U64, true); else NSORT_TSK64(DT_U64, false); }
-  else if (dt == DT_I64) { if (final_pass) NSORT_TSK64(DT_I64, true); else NSORT_TSK64(DT_I64, false); }
-  else { if (final_pass) NSORT_TSK64(DT_F64, true); else NSORT_TSK64(DT_F64, false); }
+#define NSORT_TSK64(DT)                                                                 \
+  tile_sort_keys64_kernel<KEYS64_SORT_NT, DT><<<grid, KEYS64_SORT_NT, KEYS64_SORT_SMEM, st>>>( \
+      in, out, n, samp)
+  if (dt == DT_U64) NSORT_TSK64(DT_U64);
+  else if (dt == DT_I64) NSORT_TSK64(DT_I64);
+  else NSORT_TSK64(DT_F64);
 #undef NSORT_TSK64
 }
 
@@ -1945,23 +1913,27 @@ static void launch_merge_staged64(const uint64_t *src, uint64_t *dst, int64_t n,
 int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void *tmp,
                      cudaStream_t st) {
   const Plan p = make_plan(NSORT_KIND_KEYS, (uint64_t)n, dt);
+  if (p.merge_passes == 0) {
+    TraceScope tr(TK_TILE_SORT_KEYS64, st);
+    small_sort_keys64(in, out, (int)n, dt, st);
+    return launch_status("small_sort_keys64");
+  }
   bool sorted = false;
   int rc = radix_sort_keys64(p, &sorted, in, out, dt, tmp, st);
   if (sorted || rc != NSORT_OK) return rc;
   char *t = static_cast<char *>(tmp);
-  uint64_t *bufs[2] = {out, p.merge_passes ? reinterpret_cast<uint64_t *>(t + p.keys_off) : nullptr};
-  int64_t *split = p.merge_passes ? reinterpret_cast<int64_t *>(t + p.split_off) : nullptr;
-  int *status = p.merge_passes ? reinterpret_cast<int *>(t + p.status_off) : nullptr;
-  uint64_t *samp = p.merge_passes ? reinterpret_cast<uint64_t *>(t + p.samp_off) : nullptr;
-  if (status && cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess)
+  uint64_t *bufs[2] = {out, reinterpret_cast<uint64_t *>(t + p.keys_off)};
+  int64_t *split = reinterpret_cast<int64_t *>(t + p.split_off);
+  int *status = reinterpret_cast<int *>(t + p.status_off);
+  uint64_t *samp = reinterpret_cast<uint64_t *>(t + p.samp_off);
+  if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess)
     return launch_status("cudaMemsetAsync");
   const bool tma = !(reinterpret_cast<uintptr_t>(out) & 15);
   int cur = p.merge_passes % 2;   // the last pass must land in bufs[0] == out
   const int64_t tiles = (n + p.sort_tile - 1) / p.sort_tile;
   {
     TraceScope tr(TK_TILE_SORT_KEYS64, st);
-    launch_tile_sort_keys64(in, bufs[cur], n, dt, p.merge_passes == 0, (unsigned)tiles,
-                            tma ? samp : nullptr, st);
+    launch_tile_sort_keys64(in, bufs[cur], n, dt, (unsigned)tiles, tma ? samp : nullptr, st);
   }
   rc = launch_status("tile_sort_keys64");
   for (int pass = 0; rc == NSORT_OK && pass < p.merge_passes; ++pass) {
@@ -1985,6 +1957,11 @@ int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void 
 int sort_keys_impl(const uint32_t *in, uint32_t *out, int64_t n, int dt, void *tmp,
                    cudaStream_t st) {
   const Plan p = make_plan(NSORT_KIND_KEYS, (uint64_t)n);
+  if (p.merge_passes == 0) {
+    TraceScope tr(TK_TILE_SORT_KEYS, st);
+    small_sort_keys(in, out, (int)n, dt, st);
+    return launch_status("small_sort_keys");
+  }
   int rc = NSORT_OK;
   if (p.merge4_passes == 0) {
     bool sorted = false;
@@ -1992,11 +1969,11 @@ int sort_keys_impl(const uint32_t *in, uint32_t *out, int64_t n, int dt, void *t
     if (sorted || rc != NSORT_OK) return rc;
   }
   char *t = static_cast<char *>(tmp);
-  uint32_t *bufs[2] = {out, p.merge_passes ? reinterpret_cast<uint32_t *>(t + p.keys_off) : nullptr};
-  int64_t *split = p.merge_passes ? reinterpret_cast<int64_t *>(t + p.split_off) : nullptr;
-  int *status = p.merge_passes ? reinterpret_cast<int *>(t + p.status_off) : nullptr;
-  uint32_t *samp = p.merge_passes ? reinterpret_cast<uint32_t *>(t + p.samp_off) : nullptr;
-  if (status && cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess)
+  uint32_t *bufs[2] = {out, reinterpret_cast<uint32_t *>(t + p.keys_off)};
+  int64_t *split = reinterpret_cast<int64_t *>(t + p.split_off);
+  int *status = reinterpret_cast<int *>(t + p.status_off);
+  uint32_t *samp = reinterpret_cast<uint32_t *>(t + p.samp_off);
+  if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess)
     return launch_status("cudaMemsetAsync");
   // the bulk-copy merge pass needs 16-byte aligned ping-pong buffers (the
   // scratch always is); otherwise the staged-load pass is used
@@ -2010,9 +1987,7 @@ int sort_keys_impl(const uint32_t *in, uint32_t *out, int64_t n, int dt, void *t
   const int64_t tiles = (n + p.sort_tile - 1) / p.sort_tile;
   {
     TraceScope tr(TK_TILE_SORT_KEYS, st);
-    if (p.merge_passes > 0 || !launch_small_sort(in, bufs[cur], n, dt, st))
-      launch_tile_sort_keys(in, bufs[cur], n, dt, p.merge_passes == 0, (unsigned)tiles,
-                            tma ? samp : nullptr, st);
+    launch_tile_sort_keys(in, bufs[cur], n, dt, (unsigned)tiles, tma ? samp : nullptr, st);
   }
   rc = launch_status("tile_sort_keys");
   int64_t run = p.sort_tile;
@@ -2059,6 +2034,12 @@ static int sort_pairs_typed(const uint32_t *kin, const V *vin, uint32_t *kout, V
                             int dt, void *tmp, cudaStream_t st) {
   constexpr bool V64 = sizeof(V) == 8;
   const Plan p = make_plan(V64 ? NSORT_KIND_PAIRS64 : NSORT_KIND_PAIRS, (uint64_t)n);
+  if (p.merge_passes == 0) {
+    TraceScope tr(TK_TILE_SORT_PAIRS, st);
+    if constexpr (V64) small_sort_pairs64(kin, vin, kout, vout, (int)n, dt, st);
+    else small_sort_pairs(kin, vin, kout, vout, (int)n, dt, st);
+    return launch_status("small_sort_pairs");
+  }
   bool sorted = false;
   int rc;
   if constexpr (V64) rc = radix_sort_pairs64(p, &sorted, kin, vin, kout, vout, dt, tmp, st);
@@ -2067,12 +2048,12 @@ static int sort_pairs_typed(const uint32_t *kin, const V *vin, uint32_t *kout, V
   rc = ensure_pairs_smem_attr<V>();
   if (rc != NSORT_OK) return rc;
   char *t = static_cast<char *>(tmp);
-  uint32_t *kb[2] = {kout, p.merge_passes ? reinterpret_cast<uint32_t *>(t + p.keys_off) : nullptr};
-  V *vb[2] = {vout, p.merge_passes ? reinterpret_cast<V *>(t + p.vals_off) : nullptr};
-  int64_t *split = p.merge_passes ? reinterpret_cast<int64_t *>(t + p.split_off) : nullptr;
-  int *status = p.merge_passes ? reinterpret_cast<int *>(t + p.status_off) : nullptr;
-  uint32_t *samp = p.merge_passes ? reinterpret_cast<uint32_t *>(t + p.samp_off) : nullptr;
-  if (status && cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess)
+  uint32_t *kb[2] = {kout, reinterpret_cast<uint32_t *>(t + p.keys_off)};
+  V *vb[2] = {vout, reinterpret_cast<V *>(t + p.vals_off)};
+  int64_t *split = reinterpret_cast<int64_t *>(t + p.split_off);
+  int *status = reinterpret_cast<int *>(t + p.status_off);
+  uint32_t *samp = reinterpret_cast<uint32_t *>(t + p.samp_off);
+  if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess)
     return launch_status("cudaMemsetAsync");
   // the bulk-copy merge pass needs 16-byte aligned ping-pong buffers
   const bool tma = !((reinterpret_cast<uintptr_t>(kout) | reinterpret_cast<uintptr_t>(vout)) & 15);
@@ -2080,8 +2061,8 @@ static int sort_pairs_typed(const uint32_t *kin, const V *vin, uint32_t *kout, V
   const int64_t tiles = (n + p.sort_tile - 1) / p.sort_tile;
   {
     TraceScope tr(TK_TILE_SORT_PAIRS, st);
-    launch_tile_sort_pairs<V>(kin, vin, kb[cur], vb[cur], n, dt, p.merge_passes == 0,
-                              (unsigned)tiles, tma ? samp : nullptr, st);
+    launch_tile_sort_pairs<V>(kin, vin, kb[cur], vb[cur], n, dt, (unsigned)tiles,
+                              tma ? samp : nullptr, st);
   }
   rc = launch_status("tile_sort_pairs");
   for (int pass = 0; rc == NSORT_OK && pass < p.merge_passes; ++pass) {

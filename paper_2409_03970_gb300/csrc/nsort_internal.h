@@ -43,6 +43,14 @@ int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void 
 int sort_pairs_impl(const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout,
                     int64_t n, int dt, void *tmp, cudaStream_t st);
 
+// Sorts of at most one tile, in one CTA (small.cu).
+void small_sort_keys(const uint32_t *in, uint32_t *out, int n, int dt, cudaStream_t st);
+void small_sort_keys64(const uint64_t *in, uint64_t *out, int n, int dt, cudaStream_t st);
+void small_sort_pairs(const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout,
+                      int n, int dt, cudaStream_t st);
+void small_sort_pairs64(const uint32_t *kin, const uint64_t *vin, uint32_t *kout, uint64_t *vout,
+                        int n, int dt, cudaStream_t st);
+
 // Digit sorts (radix.cu) of a plan; *sorted says whether there is one for it
 // (else nothing was done).
 int radix_sort_keys(const Plan &p, bool *sorted, const uint32_t *in, uint32_t *out, int dt,

@@ -38,37 +38,6 @@ namespace {
 
 constexpr int BINS = 256;
 
-// The order-preserving key map with the type chosen at run time by two
-// masks: to = b ^ ((b >> 31 & arith) | flip).
-template <typename K>
-struct KeyMap {
-  K arith, flip;
-};
-
-template <typename K>
-__device__ __forceinline__ K map_in(K b, KeyMap<K> m) {
-  if constexpr (sizeof(K) == 4)
-    return b ^ (((K)((int32_t)b >> 31) & m.arith) | m.flip);
-  else
-    return b ^ (((K)((int64_t)b >> 63) & m.arith) | m.flip);
-}
-
-template <typename K>
-__device__ __forceinline__ K map_out(K k, KeyMap<K> m) {
-  if constexpr (sizeof(K) == 4)
-    return k ^ (((K)((int32_t)~k >> 31) & m.arith) | m.flip);
-  else
-    return k ^ (((K)((int64_t)~k >> 63) & m.arith) | m.flip);
-}
-
-template <typename K>
-KeyMap<K> key_map(int dt) {
-  const K top = K(1) << (8 * sizeof(K) - 1);
-  if (dt == DT_F32 || dt == DT_F64) return {~K(0), top};
-  if (dt == DT_I32 || dt == DT_I64) return {K(0), top};
-  return {K(0), K(0)};
-}
-
 // ---- histograms ------------------------------------------------------------
 
 // Counts the 8-bit digits of every (mapped) key: hist[d][b] += ....  Each lane
@@ -1008,10 +977,10 @@ int radix_sort_typed(const Plan &p, bool *sorted, const K *in, const V *vin, K *
                      int dt, void *tmp, cudaStream_t st) {
   constexpr int LI = large_ipt<K>(), WI = wave_ipt<K>();
   *sorted = false;
-  // (one tile is sorted in one CTA; counts take 30 bits; 64-bit keys take
-  // eight passes, which the merge passes beat up to 1.3 million keys: 84
-  // against 109 us for 1.0e6, 114 against 126 the other way for 1.4e6)
-  if (p.merge_passes == 0 || p.n >= (int64_t(1) << 30)) return NSORT_OK;
+  // (counts take 30 bits; 64-bit keys take eight passes, which the merge
+  // passes beat up to 1.3 million keys: 84 against 109 us for 1.0e6, 114
+  // against 126 the other way for 1.4e6)
+  if (p.n >= (int64_t(1) << 30)) return NSORT_OK;
   if (sizeof(K) == 8 && p.n < 5 << 18) return NSORT_OK;
   int sms = 0;
   bool cluster = false;

@@ -76,7 +76,7 @@ struct Params {
   int *medium_list;
   int64_t *slot_base;    // large segment -> first slot of its tiles
   int *owner;            // slot -> large segment
-  uint32_t arith, flip;  // the key map of the type: b ^ ((b >> 31 & arith) | flip)
+  KeyMap<uint32_t> map;  // of the batch's type
   int dt;
   int tile;              // keys per level-0 tile: NT * 32 (keys) or NT * 16 (pairs)
   int mt;                // longest medium segment: NT * 16
@@ -89,14 +89,6 @@ __device__ __forceinline__ int ceil_log2(int64_t x) {
   int p = 0;
   while ((int64_t(1) << p) < x) ++p;
   return p;
-}
-
-// to_key and from_key of the batch's type.
-__device__ __forceinline__ uint32_t map_in(const Params &p, uint32_t b) {
-  return b ^ (((uint32_t)((int32_t)b >> 31) & p.arith) | p.flip);
-}
-__device__ __forceinline__ uint32_t map_out(const Params &p, uint32_t k) {
-  return k ^ (((uint32_t)((int32_t)~k >> 31) & p.arith) | p.flip);
 }
 
 // Entry i of medium class c's list.
@@ -273,7 +265,7 @@ struct GroupJob {
   int map;        // whether the keys are mapped back
 };
 
-// Sorts job[g], as group g of W warps of the CTA (sort_group32).  Every
+// Sorts job[g], as group g of W warps of the CTA (sort_group).  Every
 // thread of the group calls it, after thread 0 of the group wrote the job.
 // Bound by the integer ALU pipe like the plain tile sort.  A segment costs
 // as many warps as it fills (whole 16384-key tiles and power-of-two blocks
@@ -283,7 +275,7 @@ struct GroupJob {
 // tile sort; 30,000 segments up to 20,000 long 557 us in all, 790 before.
 template <int W>
 __device__ __forceinline__ void group_sort(const Params &p, void *smem, GroupJob *job, int g) {
-  uint32_t *s = static_cast<uint32_t *>(smem) + g * (W * GROUP_WARP_WORDS);
+  uint32_t *s = static_cast<uint32_t *>(smem) + g * (W * group_warp_words(32));
   const int tid = threadIdx.x & (32 * W - 1);
   auto bar = [&] {
     if constexpr (W == 1) __syncwarp();
@@ -299,19 +291,18 @@ __device__ __forceinline__ void group_sort(const Params &p, void *smem, GroupJob
     const uint32_t *in = j->in + c0;
     aw = (j->count + 1023) >> 10;
 #pragma unroll
-    for (int k = 0; k < 32; ++k) r[k] = 32 * k < left ? map_in(p, in[32 * k]) : 0xFFFFFFFFu;
+    for (int k = 0; k < 32; ++k) r[k] = 32 * k < left ? map_in(in[32 * k], p.map) : 0xFFFFFFFFu;
   }
-  sort_group32<W, Best32Columns>(r, s, tid, aw, bar);
+  sort_group<32, W, Best32Columns>(r, s, tid, aw, bar);
   // thread t holds keys [32t, 32t + 32): staged in shared memory (padded,
   // conflict-free both ways) so that the global stores are coalesced
   // whatever the segment's alignment
   bar();   // every thread is done reading s in the last merge level
   if ((tid >> 5) < aw) {
     const int pb = pidx<uint32_t>(tid * 32);
-    const uint32_t arith = j->map ? p.arith : 0u, flip = j->map ? p.flip : 0u;
+    const KeyMap<uint32_t> map = j->map ? p.map : KeyMap<uint32_t>{0u, 0u};
 #pragma unroll
-    for (int k = 0; k < 32; ++k)
-      s[pb + k] = r[k] ^ (((uint32_t)((int32_t)~r[k] >> 31) & arith) | flip);
+    for (int k = 0; k < 32; ++k) s[pb + k] = map_out(r[k], map);
   }
   bar();
   const int left = j->count - c0;
@@ -341,7 +332,7 @@ __device__ __forceinline__ void pairs_sort(const Params &p, void *smem, volatile
     m = (j->count + 511) & ~511;
 #pragma unroll
     for (int k = 0; k < 16; ++k)
-      r[k] = 32 * k < left ? make_elem<uint64_t>(map_in(p, in[32 * k]), c0 + 32 * k) : ~0ull;
+      r[k] = 32 * k < left ? make_elem<uint64_t>(map_in(in[32 * k], p.map), c0 + 32 * k) : ~0ull;
 #pragma unroll
     for (int k = 0; k < 16; ++k)
       if (32 * k < left) to[33 * k] = vin[32 * k];
@@ -355,12 +346,11 @@ __device__ __forceinline__ void pairs_sort(const Params &p, void *smem, volatile
   static_assert(2 * padded_len<uint32_t>(NT * 16) <= 2 * merge_smem_len<uint64_t>(NT * 16, 16),
                 "keys and payloads fit where the composites were");
   if (tid * 16 < m) {
-    const uint32_t arith = j->map ? p.arith : 0u, flip = j->map ? p.flip : 0u;
+    const KeyMap<uint32_t> map = j->map ? p.map : KeyMap<uint32_t>{0u, 0u};
     const int pb = pidx<uint32_t>(tid * 16);   // one pad block holds all 16
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
-      const uint32_t key = elem_key(r[k]);
-      sk[pb + k] = key ^ (((uint32_t)((int32_t)~key >> 31) & arith) | flip);
+      sk[pb + k] = map_out(elem_key(r[k]), map);
       so[pb + k] = sv[pidx<uint32_t>(elem_pos(r[k]) & (NT * 16 - 1))];
     }
   }
@@ -406,7 +396,7 @@ __device__ void warp_sort_segment(const Params &p, int64_t sid) {
 #pragma unroll
   for (int k = 0; k < IPT; ++k) {
     const int e = lane + 32 * k;
-    r[k] = e < L ? make_elem<K>(map_in(p, p.kin[off + e]), e) : (K)~(K)0;
+    r[k] = e < L ? make_elem<K>(map_in(p.kin[off + e], p.map), e) : (K)~(K)0;
   }
   column_sort(r);
   warp_merge<IPT>(r, lane);
@@ -420,7 +410,7 @@ __device__ void warp_sort_segment(const Params &p, int64_t sid) {
 #pragma unroll
   for (int k = 0; k < IPT; ++k) {
     if (e0 + k < L) {
-      p.kout[off + e0 + k] = map_out(p, elem_key(r[k]));
+      p.kout[off + e0 + k] = map_out(elem_key(r[k]), p.map);
       if (PAIRS) p.vout[off + e0 + k] = vo[k];
     }
   }
@@ -435,7 +425,7 @@ __device__ void thread_sort_segment(const Params &p, int64_t sid) {
   K r[W];
 #pragma unroll
   for (int k = 0; k < W; ++k)
-    r[k] = k < L ? make_elem<K>(map_in(p, p.kin[off + k]), k) : (K)~(K)0;
+    r[k] = k < L ? make_elem<K>(map_in(p.kin[off + k], p.map), k) : (K)~(K)0;
   column_sort(r);
   uint32_t vo[W];
   if (PAIRS) {
@@ -445,7 +435,7 @@ __device__ void thread_sort_segment(const Params &p, int64_t sid) {
 #pragma unroll
   for (int k = 0; k < W; ++k) {
     if (k < L) {
-      p.kout[off + k] = map_out(p, elem_key(r[k]));
+      p.kout[off + k] = map_out(elem_key(r[k]), p.map);
       if (PAIRS) p.vout[off + k] = vo[k];
     }
   }
@@ -574,7 +564,7 @@ size_t smem_bytes() {
   if (PAIRS)
     return sizeof(uint64_t) * merge_smem_len<uint64_t>(NT * 16, 16) +
            sizeof(uint32_t) * padded_len<uint32_t>(NT * 16);
-  return sizeof(uint32_t) * (NT / 32) * GROUP_WARP_WORDS;
+  return sizeof(uint32_t) * (NT / 32) * group_warp_words(32);
 }
 
 template <int NT, bool PAIRS, int MINB>
@@ -668,8 +658,7 @@ int segmented_impl(const void *d_keys_in, void *d_keys_out, const uint32_t *d_va
   p.medium_list = reinterpret_cast<int *>(t + l.medium);
   p.slot_base = reinterpret_cast<int64_t *>(t + l.slot);
   p.owner = reinterpret_cast<int *>(t + l.owner);
-  p.arith = dtype == NSORT_F32 ? ~0u : 0u;
-  p.flip = dtype == NSORT_U32 ? 0u : 0x80000000u;
+  p.map = key_map<uint32_t>(dtype);
   p.dt = dtype;
   p.nt = cfg.block_threads;
   p.mt = cfg.block_threads * 16;

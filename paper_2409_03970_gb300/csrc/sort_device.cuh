@@ -62,6 +62,37 @@ __device__ __forceinline__ uint64_t from_key(uint64_t k, int dt) {
   return k ^ m;
 }
 
+// The order-preserving key map with the type chosen at run time by two
+// masks: to = b ^ ((b >> 31 & arith) | flip).
+template <typename K>
+struct KeyMap {
+  K arith, flip;
+};
+
+template <typename K>
+__device__ __forceinline__ K map_in(K b, KeyMap<K> m) {
+  if constexpr (sizeof(K) == 4)
+    return b ^ (((K)((int32_t)b >> 31) & m.arith) | m.flip);
+  else
+    return b ^ (((K)((int64_t)b >> 63) & m.arith) | m.flip);
+}
+
+template <typename K>
+__device__ __forceinline__ K map_out(K k, KeyMap<K> m) {
+  if constexpr (sizeof(K) == 4)
+    return k ^ (((K)((int32_t)~k >> 31) & m.arith) | m.flip);
+  else
+    return k ^ (((K)((int64_t)~k >> 63) & m.arith) | m.flip);
+}
+
+template <typename K>
+inline KeyMap<K> key_map(int dt) {
+  const K top = K(1) << (8 * sizeof(K) - 1);
+  if (dt == DT_F32 || dt == DT_F64) return {~K(0), top};
+  if (dt == DT_I32 || dt == DT_I64) return {K(0), top};
+  return {K(0), K(0)};
+}
+
 // Shared-memory index with one pad word per 32 (u32) or per 16 (u64)
 // elements: a thread writing 16 consecutive elements and a warp reading
 // consecutive elements are both free of bank conflicts.
@@ -662,54 +693,70 @@ __device__ __forceinline__ void sort_tile_in_block(K (&r)[IPT], K *s) {
 }
 
 // ---- sort by a group of warps ----------------------------------------------
-// Words of shared memory per warp of a group sort: 1024 keys and the gap
-// behind them, padded, or the warp's transpose buffer.
-constexpr int GROUP_WARP_WORDS = 1124;
-static_assert(GROUP_WARP_WORDS >= 32 * 33 &&
-                  16 * GROUP_WARP_WORDS >= padded_len<uint32_t>(16 * (1024 + 64)),
-              "a group's runs, gaps and transposes fit");
+// Words of shared memory per warp of a group sort with IPT keys a thread: its
+// 32 IPT keys and the gap behind them, padded (at 32 keys a thread also the
+// warp's transpose buffer).
+template <typename K = uint32_t>
+__host__ __device__ constexpr int group_warp_words(int ipt) {
+  return padded_len<K>(32 * ipt + block_gap<K>(ipt));
+}
+static_assert(group_warp_words(32) >= 32 * 33, "a warp's transpose fits");
 
-// sort_tile_in_block for 32-bit keys, by the first `aw` of a group of W warps
-// (32 keys a thread, tid = thread in the group): sorts the 1024 aw keys in
-// their registers, so that thread t < 32 aw ends with keys 32 t .. 32 t + 31.
-// Only the warps that hold keys take part in the work; all W meet at the
-// barriers (bar), and s is the group's W * GROUP_WARP_WORDS words.  The last
-// run of a level may be short or have no partner (its keys stay where they
-// are).
-template <int W, class COLS, class BAR>
-__device__ __forceinline__ void sort_group32(uint32_t (&r)[32], uint32_t *s, int tid, int aw,
-                                             BAR bar) {
-  constexpr int GAP = block_gap<uint32_t>(32);
+// sort_tile_in_block (gapped: keys, or distinct composites) by the first `aw`
+// of a group of W warps
+// (tid = thread in the group): sorts the 32 IPT aw keys in their registers,
+// so that thread t < 32 aw ends with keys IPT t .. IPT (t + 1) - 1.  Only the
+// warps that hold keys take part in the work; all W meet at the barriers
+// (bar), and s is the group's W * group_warp_words(IPT) words.  The last run
+// of a level may be short or have no partner (its keys stay where they are).
+template <int IPT, int W, class COLS, typename K, class BAR>
+__device__ __forceinline__ void sort_group(K (&r)[IPT], K *s, int tid, int aw, BAR bar) {
+  constexpr int GAP = block_gap<K>(IPT);
+  constexpr int LOG0 = IPT == 32 ? 10 : (IPT == 16 ? 9 : 8);   // a warp's run
+  static_assert(32 * IPT == 1 << LOG0, "8, 16 or 32 keys a thread");
   const int lane = tid & 31;
   const bool on = (tid >> 5) < aw;
   if (on) {
     COLS::sort(r);
-    uint32_t *t = s + (tid >> 5) * (32 * 33);
-    warp_merge_level<1>(r, lane);
-    warp_merge_level<2>(r, lane);
-    warp_merge_level_t<3>(r, lane, t);
-    warp_merge_level_t<4>(r, lane, t);
-    warp_merge_level_t<5>(r, lane, t);
+    if constexpr (IPT == 32) {
+      static_assert(sizeof(K) == 4, "32 keys a thread: 32-bit ones");
+      uint32_t *t = s + (tid >> 5) * (32 * 33);
+      warp_merge_level<1>(r, lane);
+      warp_merge_level<2>(r, lane);
+      warp_merge_level_t<3>(r, lane, t);
+      warp_merge_level_t<4>(r, lane, t);
+      warp_merge_level_t<5>(r, lane, t);
+    } else if constexpr (IPT == 16 && sizeof(K) == 8) {
+      K *t = s + (tid >> 5) * 512;
+      warp_merge_level<1>(r, lane);
+      warp_merge_level16_t<2>(r, lane, t);
+      warp_merge_level16_t<3>(r, lane, t);
+      warp_merge_level16_t<4>(r, lane, t);
+      warp_merge_level16_5t(r, lane, t);
+    } else {
+      warp_merge<IPT>(r, lane);
+    }
   }
   if (W == 1 || aw == 1) return;
-  const int act = 1024 * aw;
-  const int e0 = tid * 32;
+  const int act = 32 * IPT * aw;
+  const int e0 = tid * IPT;
   // this thread's keys into the gapped layout of runs of 2^lr, and the
   // largest keys behind a run that ends with this warp's
   auto stage = [&](int lr) {
-    const int pb = pidx<uint32_t>(e0 + (e0 >> lr) * GAP);   // one pad block holds all 32
+    const int pb = pidx<K>(e0 + (e0 >> lr) * GAP);   // one pad block holds all IPT
 #pragma unroll
-    for (int k = 0; k < 32; ++k) s[pb + k] = r[k];
-    const int wend = e0 + (32 - lane) * 32;   // end of the warp's keys (same in every lane)
+    for (int k = 0; k < IPT; ++k) s[pb + k] = r[k];
+    const int wend = e0 + (32 - lane) * IPT;   // end of the warp's keys (same in every lane)
     if (!(wend & ((1 << lr) - 1)) || wend == act) {
       const int gap0 = wend + ((wend - 1) >> lr) * GAP;
-      for (int j = lane; j < GAP; j += 32) s[pidx<uint32_t>(gap0 + j)] = ~0u;
+      for (int j = lane; j < GAP; j += 32) s[pidx<K>(gap0 + j)] = ~K(0);
     }
   };
-  bar();   // every warp is done with its transpose buffer
-  if (on) stage(10);
+  if (IPT == 32 || (IPT == 16 && sizeof(K) == 8))
+    bar();   // every warp is done with its transpose buffer
+  if (on) stage(LOG0);
 #pragma unroll 1
-  for (int lr = 10; (1 << lr) < act; ++lr) {
+  for (int lr = LOG0; (1 << lr) < act; ++lr) {
     bar();
     const int run = 1 << lr;
     const int g0 = e0 & ~(2 * run - 1);
@@ -720,7 +767,7 @@ __device__ __forceinline__ void sort_group32(uint32_t (&r)[32], uint32_t *s, int
       const int a0 = g0 + (g0 >> lr) * GAP;   // run 2p and its gap, then run 2p+1
       const int b0 = a0 + run + GAP;
       const int ai = merge_path_smem(s, a0, run, b0, nb, diag);
-      serial_merge_gapped<32>(s, a0 + ai, b0 + diag - ai, r);
+      serial_merge_gapped<IPT>(s, a0 + ai, b0 + diag - ai, r);
     }
     if (2 * run < act) {
       bar();
