@@ -66,6 +66,8 @@ class NsortError(RuntimeError):
 
 def _load():
     global _lib
+    if _lib is not None:      # (set once, complete)
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -173,10 +175,28 @@ def _ptr(x) -> int:
     return x.data_ptr()
 
 
+_current_stream = None
+
+
+def _find_current_stream():
+    """How the current stream of the current device is found: by its raw
+    handle where torch offers that (0.2 us; a Stream object takes 2), else
+    through the Stream object."""
+    global _current_stream
+    import torch
+    torch.cuda.init()
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is not None and device is not None:
+        _current_stream = lambda: raw(device())                                # noqa: E731
+    else:
+        _current_stream = lambda: torch.cuda.current_stream().cuda_stream      # noqa: E731
+    return _current_stream
+
+
 def _stream(stream) -> int:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return (_current_stream or _find_current_stream())()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
