@@ -265,13 +265,19 @@ struct DigitTile {
     return free_order ? cnt + lane : cnt + warp * 2 * BINS + (lane >> 4);
   }
 
-  // Counts the digits; the counters were cleared before the last barrier of
-  // the caller or are cleared before the first one here.
+  // Counts the digits.  CLEAR: the counters were cleared before the caller's
+  // last barrier; FIRST: no digit is sorted yet, so that order is free.
+  template <bool CLEAR, bool FIRST>
   __device__ __forceinline__ void count_digits(const K (&r)[IPT]) {
-    if (tid == 0) sh.ends[0] = r[0];
-    if (tid == NT - 1) sh.ends[1] = r[IPT - 1];
-    __syncthreads();   // the counters are clear
-    free_order = !PAIRS && count == TILE && !((sh.ends[0] ^ sh.ends[1]) & low);
+    if constexpr (PAIRS || FIRST) {
+      free_order = !PAIRS && count == TILE;
+      if (!CLEAR) __syncthreads();
+    } else {
+      if (tid == 0) sh.ends[0] = r[0];
+      if (tid == NT - 1) sh.ends[1] = r[IPT - 1];
+      __syncthreads();   // (and the counters are clear)
+      free_order = count == TILE && !((sh.ends[0] ^ sh.ends[1]) & low);
+    }
     uint32_t *mine = my_counters();
     const uint32_t stride = free_order ? COPIES : 2;
 #pragma unroll
@@ -288,11 +294,27 @@ struct DigitTile {
     return free_order ? cnt + d * COPIES + ((d & (COPIES - 1)) ^ ((tid & 1) * 16) ^ j)
                       : cnt + j * 2 * BINS + tid;
   }
+  // Whether the 16 counters stay in registers between half_count and
+  // place_counters, two a word (a half-warp or a lane counts at most 512
+  // keys).  Where the registers allow it (2.0e7 int64 keys 829 -> 805 us, 2^27
+  // pairs 2.48 -> 2.43 ms); 32-bit keys and 64-bit payloads read them again
+  // (2^28 u32 keys 2.78 -> 2.85 ms with them kept).
+  static constexpr bool KEEP = sizeof(K) == 8 || (PAIRS && sizeof(V) == 4);
+  static constexpr int NKEPT = KEEP ? 8 : 1;
   // This thread's half of digit tid >> 1's count.
-  __device__ __forceinline__ uint32_t half_count() const {
+  __device__ __forceinline__ uint32_t half_count(uint32_t (&kept)[NKEPT]) const {
     uint32_t own = 0;
+    if constexpr (KEEP) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const uint32_t a = *counter(2 * j), b = *counter(2 * j + 1);
+        kept[j] = a | b << 16;
+        own += a + b;
+      }
+    } else {
 #pragma unroll 8
-    for (int j = 0; j < 16; ++j) own += *counter(j);
+      for (int j = 0; j < 16; ++j) own += *counter(j);
+    }
     return own;
   }
 
@@ -313,14 +335,25 @@ struct DigitTile {
 
   // Counts -> positions in the tile, given the digit's place in it and what
   // of its count precedes this thread's half.
-  __device__ __forceinline__ void place_counters(uint32_t run) const {
+  __device__ __forceinline__ void place_counters(uint32_t run,
+                                                 const uint32_t (&kept)[NKEPT]) const {
     const int up = free_order ? 0 : 16;
+    if constexpr (KEEP) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        *counter(2 * j) = run << up;
+        run += kept[j] & 0xFFFFu;
+        *counter(2 * j + 1) = run << up;
+        run += kept[j] >> 16;
+      }
+    } else {
 #pragma unroll 8
-    for (int j = 0; j < 16; ++j) {
-      uint32_t *c = counter(j);
-      const uint32_t v = *c;
-      *c = run << up;
-      run += v;
+      for (int j = 0; j < 16; ++j) {
+        uint32_t *c = counter(j);
+        const uint32_t v = *c;
+        *c = run << up;
+        run += v;
+      }
     }
     __syncthreads();
   }
@@ -504,13 +537,21 @@ __device__ __forceinline__ uint32_t load_of_cta(const uint32_t *p, uint32_t c) {
 // the stable passes (26 wavefronts for 32 keys, 80% of the pipe's peak; 197
 // and 211 us), and in the free-order passes (15 wavefronts, 60%; 165 us)
 // the latency of the phases of the two tiles an SM holds at a time.  A pass
-// over 2^28 keys takes 0.70 ms on average, 3.1 TB/s of keys; 2^28 keys sort
-// in 2.98 ms against 6.42 ms by merge passes, 2^27 f32 pairs in 2.49 against
-// 7.19 ms, 3.0e7 pairs with 64-bit payloads in 1.00 against 2.03 ms, 2.0e7
-// int64 keys in 0.88 against 1.07 ms.  Tried and slower at 2^28 keys: CTAs
-// that stay for several tiles and load the next one early (3.0 to 5.2 ms:
+// over 2^28 keys takes 0.65 ms on average, 3.3 TB/s of keys; 2^28 keys sort
+// in 2.78 ms against 6.42 ms by merge passes, 2^27 f32 pairs in 2.43 against
+// 7.19 ms, 3.0e7 pairs with 64-bit payloads in 0.96 against 2.03 ms, 2.0e7
+// int64 keys in 0.81 against 1.07 ms.  Tried and slower at 2^28 keys: CTAs
+// that stay for several tiles and load the next one early (2.9 to 5.2 ms:
 // tickets taken early delay the counts that later tiles wait for), one CTA
-// that scans all tiles' counts (4.35 ms), 32 tiles a look-back step (3.48).
+// that scans all tiles' counts (4.35 ms), 32 tiles a look-back step (3.48),
+// the look-back's first loads among the ranking (2.80).
+//
+// In a walk each CTA also asks L2 for the keys of the tile that starts about
+// when this one ends.  Two tiles an SM run at once, so AHEAD tiles on is well
+// before it runs and well within L2: 2^28 keys take 3.00 ms without, 2.96 with
+// 20 tiles, 2.80 with 50, 2.79 with 76 to 304, 2.93 with 608 (40 MB ahead, in
+// L2 beside the scattered writes).
+constexpr uint32_t AHEAD = 76;   // tiles: a quarter of those that run at once
 template <typename K, typename V, int IPT, bool FIRST, bool LAST, bool WAVE, int CL = 1>
 __global__ void __launch_bounds__(NT, 2) radix_pass_kernel(
     const K *__restrict__ src, const V *__restrict__ vsrc, K *__restrict__ dst,
@@ -545,14 +586,21 @@ __global__ void __launch_bounds__(NT, 2) radix_pass_kernel(
   K r[IPT];
   t.template load<false>(src + base, r);
   t.prefetch(vsrc + base);
+  if constexpr (!WAVE) {   // the keys of the tile that starts when this one ends
+    constexpr uint32_t LINE = 128 / sizeof(K);
+    const uint32_t e = base + AHEAD * T::TILE + tid * LINE;
+    static_assert(T::TILE == NT * LINE, "a line a thread");
+    if (e < n) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + e));
+  }
   if (FIRST) {
 #pragma unroll
     for (int i = 0; i < IPT; ++i) r[i] = map_in(r[i], map_i);
   }
   t.pad(r);
-  t.count_digits(r);
+  t.template count_digits<true, FIRST && !LAST>(r);   // (WAVE: FIRST and LAST are set in all passes)
   const int d = tid >> 1;
-  const uint32_t own = t.half_count();
+  uint32_t kept[T::NKEPT];
+  const uint32_t own = t.half_count(kept);
   const uint32_t other = __shfl_xor_sync(0xffffffffu, own, 1);
   const uint32_t total = own + other;
   const uint32_t flip = parity | parity >> 16;   // (WAVE) both halves' parity bits
@@ -570,7 +618,7 @@ __global__ void __launch_bounds__(NT, 2) radix_pass_kernel(
   if constexpr (CL > 1) cluster_arrive();   // the count is there for the other CTAs
   const uint32_t tbase = t.sum_below(total);   // where the digit starts in the tile
   if (!(tid & 1)) sh.tile_base[d] = tbase;
-  t.place_counters(tbase + (tid & 1 ? other : 0u));
+  t.place_counters(tbase + (tid & 1 ? other : 0u), kept);
   [[maybe_unused]] uint32_t excl0 = 0;   // (WAVE) all smaller digits, and the cluster's lower ranks
   if constexpr (WAVE) excl0 = t.sum_below(hist[d]);
   if constexpr (CL > 1) {
@@ -742,12 +790,13 @@ __global__ void __launch_bounds__(NT, 1) radix_cluster_kernel(
       for (int i = 0; i < IPT; ++i) r[i] = map_in(r[i], map);
     }
     t.pad(r);
-    t.count_digits(r);
-    const uint32_t own = t.half_count();
+    t.template count_digits<false, false>(r);
+    uint32_t kept[T::NKEPT];
+    const uint32_t own = t.half_count(kept);
     const uint32_t other = __shfl_xor_sync(0xffffffffu, own, 1);
     if (!(tid & 1)) sh.tile_total[d] = own + other;
     const uint32_t tbase = t.sum_below(own + other);
-    t.place_counters(tbase + (tid & 1 ? other : 0u));
+    t.place_counters(tbase + (tid & 1 ? other : 0u), kept);
     cluster_arrive();   // this CTA's counts are there
     uint32_t pos2[T::NPOS];
     t.rank(r, pos2);
