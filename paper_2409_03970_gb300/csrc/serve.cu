@@ -10,9 +10,10 @@
 // completion event, once no smaller request waits):
 // large requests run alone as nsort_keys / nsort_pairs; small ones
 // (n <= batch_max_keys) are co-batched with the other waiting small requests
-// of the same kind and dtype into one segmented sort (a gather kernel packs
-// their keys, nsort_segmented sorts every request as its own segment, a
-// scatter kernel writes each result back).  Admitted work on different slots
+// of the same kind and dtype into one segmented sort (a copy kernel packs
+// their keys, nsort_segmented sorts every request as its own segment, the
+// copy kernel writes each result back); one that finds no other to join runs
+// as the plain call too.  Admitted work on different slots
 // overlaps on the device.  Completion is signalled from the stream by a host
 // function; the scheduler then frees the scratch and wakes waiters.  Each
 // result is bit-identical to the plain call on the same input, batched or
@@ -54,27 +55,85 @@ struct BatchItem {
   int64_t n;
 };
 
-// Packs every request of a batch into one array (keys and values).
-__global__ void batch_gather_kernel(const BatchItem *items, int count, uint32_t *sk, uint32_t *sv) {
-  for (int i = blockIdx.x; i < count; i += gridDim.x) {
-    const BatchItem it = items[i];
-    for (int64_t e = threadIdx.x; e < it.n; e += blockDim.x) {
-      sk[it.off + e] = it.kin[e];
-      if (sv) sv[it.off + e] = it.vin[e];
-    }
+// The last of the items lo .. hi that begins at or before e (none is empty,
+// offs[lo] <= e).
+__device__ __forceinline__ int item_at(const int64_t *offs, int lo, int hi, int64_t e) {
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (offs[mid] <= e)
+      lo = mid;
+    else
+      hi = mid - 1;
   }
+  return lo;
 }
 
-// Writes each request's sorted segment back to its own output.
-__global__ void batch_scatter_kernel(const BatchItem *items, int count, const uint32_t *sk,
-                                     const uint32_t *sv) {
-  for (int i = blockIdx.x; i < count; i += gridDim.x) {
-    const BatchItem it = items[i];
-    for (int64_t e = threadIdx.x; e < it.n; e += blockDim.x) {
-      it.kout[e] = sk[it.off + e];
-      if (sv) it.vout[e] = sv[it.off + e];
+// PACK: packs every request of a batch into one array (keys and values);
+// else writes each request's sorted segment back to its own output.  A copy,
+// bound by latency at the sizes that are batched (a few dependent loads to
+// find the request, then one load and one store).  So the packed array is cut
+// into chunks of four keys a thread, whatever requests they belong to: with a
+// CTA per request, one of 65,536 keys took 256 rounds of load and store in a
+// row, and a co-batch with one in it 245-300 us from admission to completion
+// (in a burst of 32 requests of 1,406 to 3.2 million keys); now 120-150.
+constexpr int COPY_NT = 256, COPY_PER = 4, COPY_CHUNK = COPY_NT * COPY_PER;
+template <bool PACK>
+__global__ void __launch_bounds__(COPY_NT) batch_copy_kernel(const BatchItem *items,
+                                                             const int64_t *offs, int count,
+                                                             uint32_t *sk, uint32_t *sv) {
+  const int64_t total = offs[count];
+  const int64_t first = (int64_t)blockIdx.x * COPY_CHUNK;
+  if (first >= total) return;
+  const int64_t last = (total < first + COPY_CHUNK ? total : first + COPY_CHUNK) - 1;
+  const int lo = item_at(offs, 0, count - 1, first);
+  const int hi = item_at(offs, lo, count - 1 < lo + COPY_CHUNK ? count - 1 : lo + COPY_CHUNK, last);
+  const uint32_t *from[COPY_PER], *vfrom[COPY_PER];
+  uint32_t *to[COPY_PER], *vto[COPY_PER];
+#pragma unroll
+  for (int j = 0; j < COPY_PER; ++j) {
+    const int64_t e = first + j * COPY_NT + threadIdx.x;
+    if (e > last) continue;
+    const BatchItem *it = items + item_at(offs, lo, hi, e);
+    const int64_t at = e - it->off;
+    from[j] = PACK ? it->kin + at : sk + e;
+    to[j] = PACK ? sk + e : it->kout + at;
+    if (sv) {
+      vfrom[j] = PACK ? it->vin + at : sv + e;
+      vto[j] = PACK ? sv + e : it->vout + at;
     }
   }
+  uint32_t k[COPY_PER], v[COPY_PER];
+#pragma unroll
+  for (int j = 0; j < COPY_PER; ++j)
+    if (first + j * COPY_NT + threadIdx.x <= last) {
+      k[j] = *from[j];
+      if (sv) v[j] = *vfrom[j];
+    }
+#pragma unroll
+  for (int j = 0; j < COPY_PER; ++j)
+    if (first + j * COPY_NT + threadIdx.x <= last) {
+      *to[j] = k[j];
+      if (sv) *vto[j] = v[j];
+    }
+}
+
+// Whether a request that may be co-batched, alone in its batch, can be sorted
+// by the plain call: the scratch of the batch suffices for it, and nothing
+// that it writes is read, or written, through another of its pointers (in a
+// batch everything is read before anything is written).  The plain call needs
+// neither the descriptors nor the two copies nor the segmented sort's set-up:
+// 57,525 keys take 75 us from admission to completion, 245 before.  The burst
+// of 32 took 1226 us, 691 with both.
+bool plain_alone(const nsort_request &r, size_t scratch) {
+  if (nsort_temp_bytes(r.kind, r.n, 0, r.dtype) > scratch) return false;
+  auto apart = [&](const void *a, const void *b) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x + r.n * 4 <= y || y + r.n * 4 <= x;
+  };
+  if (!apart(r.d_keys_in, r.d_keys_out)) return false;
+  if (r.kind == NSORT_KIND_KEYS) return true;
+  return apart(r.d_vals_in, r.d_vals_out) && apart(r.d_keys_in, r.d_vals_out) &&
+         apart(r.d_vals_in, r.d_keys_out) && apart(r.d_keys_out, r.d_vals_out);
 }
 
 double now_s() {
@@ -181,8 +240,10 @@ void launch(Ctx *c, int s, std::vector<Pending> &picked, std::vector<std::pair<s
   for (auto &p : picked) c->reqs[p.ticket].t_admit = t;
   int rc = NSORT_OK;
   if (after && cudaStreamWaitEvent(slot.stream, after, 0) != cudaSuccess) rc = NSORT_ECUDA;
-  if (picked.size() == 1 && c->reqs[picked[0].ticket].batched == 0) {
-    const Req &q = c->reqs[picked[0].ticket];
+  const Req &head = c->reqs[picked[0].ticket];
+  if (picked.size() == 1 &&
+      (head.batched == 0 || plain_alone(head.r, allocs[0].second))) {
+    const Req &q = head;
     void *tmp = allocs.empty() ? nullptr : c->arena_base + allocs[0].first;
     const size_t tb = allocs.empty() ? 0 : allocs[0].second;
     if (q.r.kind == NSORT_KIND_KEYS)
@@ -233,14 +294,14 @@ void launch(Ctx *c, int s, std::vector<Pending> &picked, std::vector<std::pair<s
         cudaSuccess)
       rc = NSORT_ECUDA;
     if (rc == NSORT_OK) {
-      const unsigned g = (unsigned)(count < 2048 ? count : 2048);
-      batch_gather_kernel<<<g, 256, 0, slot.stream>>>(items, (int)count, sk, sv);
+      const unsigned g = (unsigned)((total + COPY_CHUNK - 1) / COPY_CHUNK);
+      batch_copy_kernel<true><<<g, COPY_NT, 0, slot.stream>>>(items, offs, (int)count, sk, sv);
       // no segment is longer than the longest request: launch only the
       // merge levels it needs
       rc = segmented_impl(sk, sk, sv, sv, offs, count, total, picked[0].dtype, segtmp, segbytes,
                           slot.stream, longest);
       if (rc == NSORT_OK) {
-        batch_scatter_kernel<<<g, 256, 0, slot.stream>>>(items, (int)count, sk, sv);
+        batch_copy_kernel<false><<<g, COPY_NT, 0, slot.stream>>>(items, offs, (int)count, sk, sv);
         if (cudaGetLastError() != cudaSuccess) rc = NSORT_ECUDA;
       }
     }
