@@ -773,6 +773,8 @@ __global__ void __launch_bounds__(NT, 1) radix_cluster_kernel(
   const uint32_t rank = cluster_rank();
   const uint32_t base = rank * (uint32_t)T::TILE;
   t.count = base >= n ? 0u : (n - base < (uint32_t)T::TILE ? n - base : (uint32_t)T::TILE);
+  pdl_trigger();
+  pdl_wait();
   if (rank == 0 && tid == 0) *status = NSORT_OK;
   const K *src = in;
   const V *vsrc = vin;
@@ -946,21 +948,11 @@ int radix_status(cudaError_t e, const char *what) {
 template <typename K, typename V, int IPT>
 void launch_cluster(const Plan &p, const K *in, const V *vin, K *out, V *vout, int dt, char *t,
                     cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(CLUSTER);
-  cfg.blockDim = dim3(NT);
-  cfg.dynamicSmemBytes = tile_smem<K, IPT>();
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = CLUSTER;
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
   TraceScope tr(TK_RADIX_CLUSTER, st);
-  cudaLaunchKernelEx(&cfg, radix_cluster_kernel<K, V, IPT, CLUSTER>, in, vin, out, vout,
-                     reinterpret_cast<K *>(t + p.keys_off), reinterpret_cast<V *>(t + p.vals_off),
-                     (uint32_t)p.n, key_map<K>(dt), reinterpret_cast<int *>(t + p.status_off));
+  launch_pdl<CLUSTER>(radix_cluster_kernel<K, V, IPT, CLUSTER>, CLUSTER, NT, tile_smem<K, IPT>(),
+                      st, in, vin, out, vout, reinterpret_cast<K *>(t + p.keys_off),
+                      reinterpret_cast<V *>(t + p.vals_off), (uint32_t)p.n, key_map<K>(dt),
+                      reinterpret_cast<int *>(t + p.status_off));
 }
 
 template <typename K, typename V, int IPT, bool WAVE, int CL>

@@ -13,14 +13,21 @@
 // 256 x 16 before: 1000: 12.6 / 5.5 (128 x 8), 4096: 13.0 / 13.2 (256 x 16).
 // (The larger shapes were one of 512 x 16 up to 8192 and one of 512 x 32
 // above, all of whose threads worked whatever n was.)
+//
+// They are dependent launches that let the stream's next kernel be launched
+// (and wait) as soon as they start, so that sorts that follow one another
+// don't pay for a launch each: 1000 keys 6.2 -> 4.6 us a call, back to back,
+// 1000 64-bit keys 8.4 -> 5.7, 500 pairs 8.4 -> 5.7, 10,000 keys 18.7 -> 16.5.
 #include <cuda_runtime.h>
 
 #include <atomic>
 #include <cstdint>
 
 #include "nsort.h"
+#include "launch.h"
 #include "nsort_internal.h"
 #include "sort_device.cuh"
+#include "tma_device.cuh"
 
 namespace nsort {
 
@@ -66,6 +73,8 @@ template <int W, int IPT, typename K, bool FULL = false>
 __global__ void __launch_bounds__(32 * W) small_keys_kernel(const K *in, K *out, int n,
                                                             KeyMap<K> map) {
   extern __shared__ __align__(16) unsigned char sk_smem[];   // W * group_warp_words<K>(IPT) keys
+  pdl_trigger();
+  pdl_wait();
   const int tid = threadIdx.x;
   const int c0 = (tid >> 5) * (32 * IPT) + (tid & 31);   // a warp loads 32 IPT keys in a row
   K r[IPT];
@@ -112,6 +121,8 @@ __global__ void __launch_bounds__(32 * W) small_pairs_kernel(const uint32_t *kin
                                                              uint32_t *kout, V *vout, int n,
                                                              KeyMap<uint32_t> map) {
   extern __shared__ __align__(16) unsigned char sp_smem[];
+  pdl_trigger();
+  pdl_wait();
   uint64_t *s = reinterpret_cast<uint64_t *>(sp_smem);
   V *sv = reinterpret_cast<V *>(s + W * group_warp_words<uint64_t>(IPT));   // 32 W IPT payloads
   const int tid = threadIdx.x;
@@ -160,7 +171,7 @@ void launch_keys(const K *in, K *out, int n, int dt, cudaStream_t st) {
   constexpr size_t smem = sizeof(K) * W * group_warp_words<K>(IPT);
   static_assert(W * group_warp_words<K>(IPT) >= block_smem_len<K>(32 * W, IPT), "FULL fits too");
   if (opt_in<small_keys_kernel<W, IPT, K, FULL>>(smem))
-    small_keys_kernel<W, IPT, K, FULL><<<1, 32 * W, smem, st>>>(in, out, n, key_map<K>(dt));
+    launch_pdl(small_keys_kernel<W, IPT, K, FULL>, 1, 32 * W, smem, st, in, out, n, key_map<K>(dt));
 }
 
 template <int W, int IPT, typename V>
@@ -169,8 +180,8 @@ void launch_pairs(const uint32_t *kin, const V *vin, uint32_t *kout, V *vout, in
   constexpr size_t smem = sizeof(uint64_t) * W * group_warp_words<uint64_t>(IPT) +
                           sizeof(V) * 32 * W * IPT;
   if (opt_in<small_pairs_kernel<W, IPT, V>>(smem))
-    small_pairs_kernel<W, IPT, V><<<1, 32 * W, smem, st>>>(kin, vin, kout, vout, n,
-                                                         key_map<uint32_t>(dt));
+    launch_pdl(small_pairs_kernel<W, IPT, V>, 1, 32 * W, smem, st, kin, vin, kout, vout, n,
+               key_map<uint32_t>(dt));
 }
 
 template <typename V>

@@ -44,11 +44,11 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
 // Programmatic dependent launch: blocks until the grids this one depends on
 // (the previous kernel of the stream, when this one was launched with
 // programmatic stream serialisation) have completed and their memory is
-// visible; a no-op for a plain launch.  Only the digit passes of small sorts,
-// whose tiles all run at once, trigger their dependents early (pdl_trigger):
-// else each dependent launch is released when its predecessor completes,
-// which hides the launch latency without letting the next grid's CTAs take
-// SM resources while the current grid still runs.
+// visible; a no-op for a plain launch.  Only kernels of small sorts, whose
+// CTAs all run at once, trigger their dependents early (pdl_trigger): else
+// each dependent launch is released when its predecessor completes, which
+// hides the launch latency without letting the next grid's CTAs take SM
+// resources while the current grid still runs.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel's CTAs start (and wait for this one) once every CTA
 // of this one has got here.
