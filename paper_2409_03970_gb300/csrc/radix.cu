@@ -38,6 +38,17 @@ namespace {
 
 constexpr int BINS = 256;
 
+// Sets the histograms and the tickets to zero.  A kernel and not a memset,
+// since kernels can be launched before their predecessors end: us, memset and
+// plain launch of the histograms / this: 2^20 keys 44.8 / 39.3, 3.0e6 66.0 /
+// 62.6, 200,003 pairs 35.4 / 30.8, 8.0e6 keys 131 / 125.5.  It does not release
+// the histogram kernel early: the CTAs of that would crowd on the SMs that the
+// last pass of a sort before leaves first (3.0e6: 74.7).
+__global__ void radix_init_kernel(uint32_t *words, int n) {
+  pdl_wait();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) words[i] = 0;
+}
+
 // ---- histograms ------------------------------------------------------------
 
 // Counts the 8-bit digits of every (mapped) key: hist[d][b] += ....  Each lane
@@ -45,7 +56,8 @@ constexpr int BINS = 256;
 // mod COPIES, the copies of one counter in different banks), so that equal
 // digits of a warp do not queue up on one address.  Also sets the passes'
 // look-back words to "no entry" and the status word to NSORT_OK.
-// SMALL: the first pass may start to wait early.
+// SMALL: the first pass may start to wait early (and take its tickets, which
+// are zero by then: after pdl_wait).
 template <typename K, int NT, int COPIES, bool SMALL>
 __global__ void __launch_bounds__(NT) radix_histogram_kernel(const K *__restrict__ in, int64_t n,
                                                              KeyMap<K> map, uint32_t *hist,
@@ -57,6 +69,7 @@ __global__ void __launch_bounds__(NT) radix_histogram_kernel(const K *__restrict
   for (int i = tid; i < D * BINS * COPIES; i += NT) rh_cnt[i] = 0;
   const int64_t gtid = (int64_t)blockIdx.x * NT + tid;
   const int64_t gsize = (int64_t)gridDim.x * NT;
+  pdl_wait();
   for (int64_t i = gtid; i < state_words; i += gsize) state[i] = 0xFFFFFFFFu;
   if (gtid == 0) *status = NSORT_OK;
   if (SMALL) pdl_trigger();
@@ -965,16 +978,16 @@ int radix_passes(const Plan &p, const RadixLayout &l, int sms, const K *in, cons
   K *buf = reinterpret_cast<K *>(t + p.keys_off);
   V *vbuf = reinterpret_cast<V *>(t + p.vals_off);
   const KeyMap<K> map = key_map<K>(dt), none = {K(0), K(0)};
-  const cudaError_t e = cudaMemsetAsync(hist, 0, l.state_off - l.hist_off, st);
   {
     TraceScope tr(TK_RADIX_HIST, st);
+    launch_pdl(radix_init_kernel, 1, 1024, 0, st, hist, (int)((l.state_off - l.hist_off) / 4));
     const int64_t words = (int64_t)(l.end - l.state_off) / 4;
     if constexpr (WAVE)
-      radix_histogram_kernel<K, HIST_SMALL_NT, hist_copies<K, true>(), true>
-          <<<sms, HIST_SMALL_NT, hist_smem<K, true>(), st>>>(in, p.n, map, hist, state, words, status);
+      launch_pdl(radix_histogram_kernel<K, HIST_SMALL_NT, hist_copies<K, true>(), true>, sms,
+                 HIST_SMALL_NT, hist_smem<K, true>(), st, in, p.n, map, hist, state, words, status);
     else
-      radix_histogram_kernel<K, HIST_NT, hist_copies<K, false>(), false>
-          <<<sms, HIST_NT, hist_smem<K, false>(), st>>>(in, p.n, map, hist, state, words, status);
+      launch_pdl(radix_histogram_kernel<K, HIST_NT, hist_copies<K, false>(), false>, sms, HIST_NT,
+                 hist_smem<K, false>(), st, in, p.n, map, hist, state, words, status);
   }
   const K *src = in;
   const V *vsrc = vin;
@@ -999,7 +1012,7 @@ int radix_passes(const Plan &p, const RadixLayout &l, int sms, const K *in, cons
     src = dst;
     vsrc = vdst;
   }
-  return radix_status(e, "radix pass");
+  return radix_status(cudaSuccess, "radix pass");
 }
 
 // Sorts a plan's keys by digits if there is a way to (*sorted).  The scratch of
@@ -1007,11 +1020,11 @@ int radix_passes(const Plan &p, const RadixLayout &l, int sms, const K *in, cons
 // it and by how many tiles the device runs at once.  us, merge passes against
 // digits, u32 keys / f32 pairs / pairs with 64-bit payloads:
 //   one cluster (up to 2^16, or 2^17 where the next does not fit):
-//     17,000: 28 / 40 / 43 -> 19 / 21 / 25;  65,000: 42 / 53 / 55 -> 24 / 28 / 33
+//     17,000: 28 / 40 / 43 -> 17 / 20 / 22;  65,000: 42 / 53 / 55 -> 22 / 26 / 31
 //   wave passes in clusters of four (4096-key tiles, two per SM: 1.2 million):
-//     200,003: 47 / 60 / 63 -> 32 / 35 / 40;  2^20: 63 / 80 / 108 -> 42 / 50 / 57
+//     200,003: 47 / 60 / 63 -> 29 / 31 / 36;  2^20: 63 / 80 / 108 -> 39 / 44 / 52
 //   wave passes of one CTA (10240- or 16384-key tiles: 5.0 million):
-//     3.0e6: 127 / 210 / 249 -> 68 / 87 / 139
+//     3.0e6: 127 / 210 / 249 -> 64 / 80 / 122
 //   look-back passes beyond.
 template <typename K, typename V>
 int radix_sort_typed(const Plan &p, bool *sorted, const K *in, const V *vin, K *out, V *vout,
