@@ -93,9 +93,10 @@ size_t nsort_temp_bytes(int kind, uint64_t n, uint64_t nseg, int dtype);
  * KEYS or PAIRS): one tile sort plus ceil(log2(ceil(n / tile))) global merge
  * passes.  Writes the tile sizes through the non-NULL pointers.  Used to
  * compute the algorithmic bytes of a sort (passes x 2 x element bytes x n).
- * This is the plan of the merge sort; most sorts of more than a tile (64-bit
- * keys from 1.3 million on) are done in as many stable passes over the array
- * as a key has bytes instead, with the same result and the same scratch. */
+ * This is the plan of the merge sort; most sorts of more than a tile (of
+ * 64-bit keys: of more than 655,360, but for some around a million) are done
+ * in as many stable passes over the array as a key has bytes instead, with the
+ * same result and the same scratch. */
 int nsort_plan(int kind, uint64_t n, int *passes, int *sort_tile, int *merge_tile);
 
 /* nsort_plan for keys of `dtype`: 64-bit dtypes (kind KEYS only) sort

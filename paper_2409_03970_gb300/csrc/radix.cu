@@ -902,10 +902,11 @@ bool opt_in_cluster(cudaLaunchConfig_t *cfg, int *clusters) {
          cudaOccupancyMaxActiveClusters(clusters, kernel, cfg) == cudaSuccess;
 }
 
-// What the device offers: SMs << 1 | whether a cluster of CLUSTER CTAs fits;
-// found, and the kernels of a key and payload type opted in, once per device.
+// What the device offers: how many clusters of WAVE_CL CTAs of the passes run
+// at once << 16 | SMs << 1 | whether a cluster of CLUSTER CTAs fits; found, and
+// the kernels of a key and payload type opted in, once per device.
 template <typename K, typename V>
-int radix_setup(int *sms, bool *cluster) {
+int radix_setup(int *sms, bool *cluster, int *wave_clusters) {
   static std::atomic<int> cached[64];
   int dev = 0, c = 0;
   cudaGetDevice(&dev);
@@ -920,7 +921,7 @@ int radix_setup(int *sms, bool *cluster) {
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    int least = sizeof(K) == 8 ? 0 : 1, k = 0;
+    int least = sizeof(K) == 8 ? 0 : 1, k = 0, wave = 0;
     if (!opt_in(radix_pass_kernel<K, V, LI, true, false, false>, tile_smem<K, LI>()) ||
         !opt_in(radix_pass_kernel<K, V, LI, false, false, false>, tile_smem<K, LI>()) ||
         !opt_in(radix_pass_kernel<K, V, LI, false, true, false>, tile_smem<K, LI>()) ||
@@ -942,12 +943,20 @@ int radix_setup(int *sms, bool *cluster) {
       least = k < least ? k : least;
       if (!opt_in_cluster<K, V, 16>(&cfg, &k)) return NSORT_ECUDA;
       least = k < least ? k : least;
+      cfg.gridDim = dim3(WAVE_CL);
+      cfg.dynamicSmemBytes = tile_smem<K, WAVE_CL_IPT>();
+      attr.val.clusterDim.x = WAVE_CL;
+      if (cudaOccupancyMaxActiveClusters(
+              &wave, radix_pass_kernel<K, V, WAVE_CL_IPT, true, true, true, WAVE_CL>, &cfg) !=
+          cudaSuccess)
+        return NSORT_ECUDA;
     }
-    c = *sms << 1 | (least > 0 ? 1 : 0);
+    c = wave << 16 | *sms << 1 | (least > 0 ? 1 : 0);
     if (dev < 64) cached[dev].store(c);
   }
-  *sms = c >> 1;
+  *sms = c >> 1 & 0x7FFF;
   *cluster = c & 1;
+  *wave_clusters = c >> 16;
   return NSORT_OK;
 }
 
@@ -1021,7 +1030,9 @@ int radix_passes(const Plan &p, const RadixLayout &l, int sms, const K *in, cons
 // digits, u32 keys / f32 pairs / pairs with 64-bit payloads:
 //   one cluster (up to 2^16, or 2^17 where the next does not fit):
 //     17,000: 28 / 40 / 43 -> 17 / 20 / 22;  65,000: 42 / 53 / 55 -> 22 / 26 / 31
-//   wave passes in clusters of four (4096-key tiles, two per SM: 1.2 million):
+//   wave passes in clusters of four (4096-key tiles, as many as run at once:
+//   74 on 152 SMs, 1.2 million keys; with all 76, two SMs' worth of which wait
+//   for others to end, 1.22e6 u32 keys took 61 us, 40 the next way):
 //     200,003: 47 / 60 / 63 -> 29 / 31 / 36;  2^20: 63 / 80 / 108 -> 39 / 44 / 52
 //   wave passes of one CTA (10240- or 16384-key tiles: 5.0 million):
 //     3.0e6: 127 / 210 / 249 -> 64 / 80 / 122
@@ -1031,20 +1042,25 @@ int radix_sort_typed(const Plan &p, bool *sorted, const K *in, const V *vin, K *
                      int dt, void *tmp, cudaStream_t st) {
   constexpr int LI = large_ipt<K>(), WI = wave_ipt<K>();
   *sorted = false;
-  // (counts take 30 bits; 64-bit keys take eight passes, which the merge
-  // passes beat up to 1.3 million keys: 84 against 109 us for 1.0e6, 114
-  // against 126 the other way for 1.4e6)
-  if (p.n >= (int64_t(1) << 30)) return NSORT_OK;
-  if (sizeof(K) == 8 && p.n < 5 << 18) return NSORT_OK;
-  int sms = 0;
+  if (p.n >= (int64_t(1) << 30)) return NSORT_OK;   // (counts take 30 bits)
+  // 64-bit keys take eight passes, which the merge passes beat, on sorted keys
+  // at least, outside two ranges.  int64, uniform / sorted, merges -> digits:
+  //   5.0e5: 60 / 55 -> 64 / 64;  6.6e5 (5 << 17): 77 / 69 -> 64 / 64;
+  //   9.3e5: 81 / 72 -> 70 / 70;  then a larger tile: 9.5e5: 83 / 73 -> 80 / 79,
+  //   1.1e6: 92 / 81 -> 82 / 82;  1.18e6 (9 << 17): 106 / 90 -> 84 / 83;
+  //   then two tiles an SM: 1.3e6: 120 / 104 -> 108 / 107,
+  //   2.0e6: 149 / 128 -> 132 / 131;  4.0e6: 256 / 217 -> 206 / 205.
+  if (sizeof(K) == 8 && p.n < 5 << 17) return NSORT_OK;
+  int sms = 0, wave_clusters = 0;
   bool cluster = false;
-  if (radix_setup<K, V>(&sms, &cluster) != NSORT_OK)
+  if (radix_setup<K, V>(&sms, &cluster, &wave_clusters) != NSORT_OK)
     return radix_status(cudaGetLastError(), "radix set-up");
+  if (sizeof(K) == 8 && p.n > (int64_t)sms * NT * WI && p.n < 9 << 17) return NSORT_OK;
   char *t = static_cast<char *>(tmp);
   RadixLayout l;
   if constexpr (sizeof(K) == 4) {
     l = radix_layout(p, sizeof(K), NT * WAVE_CL_IPT * WAVE_CL, true);
-    const bool wave_fits = l.end <= p.total && l.tiles * WAVE_CL <= 2 * sms;
+    const bool wave_fits = l.end <= p.total && l.tiles <= wave_clusters;
     const int64_t each = (p.n + CLUSTER * NT - 1) / (CLUSTER * NT);
     if (cluster && (each <= 8 || (each <= 16 && !wave_fits))) {
       *sorted = true;
@@ -1057,6 +1073,17 @@ int radix_sort_typed(const Plan &p, bool *sorted, const K *in, const V *vin, K *
       *sorted = true;
       return radix_passes<K, V, WAVE_CL_IPT, true, WAVE_CL>(p, l, sms, in, vin, out, vout, dt, t,
                                                             st);
+    }
+  }
+  if constexpr (std::is_same_v<V, NoValue>) {
+    // Keys alone: rather one large tile on each SM than two small ones on some
+    // and one on others, which the pass would wait for (u32, two small / one
+    // large: 1.6e6: 58.7 / 52.8, 2.4e6: 63.4 / 58.9; int64: 1.2e6: 105 / 88).  A tile's payloads take
+    // longer than that saves: 2.4e6 pairs 78.8 / 81.7, 64-bit payloads 116 / 129.
+    l = radix_layout(p, sizeof(K), NT * LI, true);
+    if (l.end <= p.total && l.tiles <= sms && p.n > (int64_t)sms * NT * WI) {
+      *sorted = true;
+      return radix_passes<K, V, LI, true, 1>(p, l, sms, in, vin, out, vout, dt, t, st);
     }
   }
   l = radix_layout(p, sizeof(K), NT * WI, true);

@@ -90,13 +90,17 @@ def sizes32(merge_tile):
     clusters = (at_once // 4) * 4 * 4096
     return [(merge_tile + 1, CLUSTER), (32768, CLUSTER), (32769, CLUSTER), (65536, CLUSTER),
             (65537, None), (131072, None), (131073, None), (200_003, PASSES),
-            (clusters, PASSES), (clusters + 1, PASSES), (at_once * 10240 + 1, PASSES),
-            (at_once * 16384 + 1, PASSES)]
+            (clusters, PASSES), (clusters + 1, PASSES), (at_once // 2 * 10240 + 1, PASSES),
+            (at_once // 2 * 16384, PASSES), (at_once // 2 * 16384 + 1, PASSES),
+            (at_once * 10240 + 1, PASSES), (at_once * 16384 + 1, PASSES)]
 
 
 def sizes64():
     at_once = 2 * torch.cuda.get_device_properties(0).multi_processor_count
-    return [((5 << 18) - 1, ["merge_keys64"]), (5 << 18, PASSES), (at_once * 6144 + 1, PASSES),
+    return [((5 << 17) - 1, ["merge_keys64"]), (5 << 17, PASSES),
+            (at_once // 2 * 6144, PASSES), (at_once // 2 * 6144 + 1, ["merge_keys64"]),
+            ((9 << 17) - 1, ["merge_keys64"]), (9 << 17, PASSES), (at_once // 2 * 8192, PASSES),
+            (at_once // 2 * 8192 + 1, PASSES), (at_once * 6144 + 1, PASSES),
             (at_once * 8192, PASSES), (at_once * 8192 + 1, PASSES), ((1 << 22) - 1, PASSES)]
 
 
