@@ -62,8 +62,8 @@ def parse():
                     help="seconds of Poisson arrivals in the served measurement (60 = the stated workload)")
     ap.add_argument("--segments", type=int, default=100_000)
     ap.add_argument("--merge-ways", type=int, choices=[2, 4], default=2,
-                    help="merge levels per pass over the array for 32-bit keys: 2 = one level "
-                         "(the library's default), 4 = two levels (four-way passes)")
+                    help="for 32-bit keys: 2 = the library's default way, 4 = merge passes of "
+                         "two levels each (four-way passes)")
     ap.add_argument("--no-numa-bind", action="store_true",
                     help="do not restrict the process to the GPU's NUMA node")
     return ap.parse_args()
@@ -467,6 +467,27 @@ def time_sort(nsort, torch, fn, reps: int = 5, warm: int = 2):
     return float(np.median(ts))
 
 
+def moved_bytes(trace, sorts: int, n: int, esize: int, vsize: int, plan_passes: int):
+    """(passes over the array, algorithmic bytes) of one sort of n keys of
+    esize and payloads of vsize bytes, from the trace of `sorts` sorts: digit
+    passes read and write everything, and one read of the keys counts their
+    digits; a sort without them ran the merge plan's passes."""
+    rp = trace.get("radix_pass")
+    if rp and rp["launches"]:
+        passes = rp["launches"] // sorts
+        return passes, (passes * 2 * (esize + vsize) + esize) * n
+    return plan_passes, plan_passes * 2 * (esize + vsize) * n
+
+
+def traced(nsort, torch, fn, reps: int = 3):
+    """The library's trace of reps calls of fn()."""
+    nsort.nsort_trace_enable(True)
+    time_sort(nsort, torch, fn, reps=reps, warm=0)
+    tr = nsort.nsort_trace_read()
+    nsort.nsort_trace_enable(False)
+    return tr
+
+
 def bench_configs(nsort, torch):
     """The other plain-sort configurations: 2^28 int32 / float32 keys over
     the five distributions (uniform, sorted, reverse, 16 distinct, Zipf), 2^27 stable float32 key / uint32 value pairs
@@ -503,23 +524,25 @@ def bench_configs(nsort, torch):
     del k, v
     kout, vout = torch.empty_like(kt), torch.empty_like(vt)
     tmp = nsort.scratch(nsort.KIND_PAIRS, m)
-    passes, _, _ = nsort.nsort_plan(nsort.KIND_PAIRS, m)
-    ms = time_sort(nsort, torch, lambda: nsort.nsort_pairs(kt, vt, kout, vout, m, nsort.F32, tmp,
-                                                           tmp.numel()))
+    plan, _, _ = nsort.nsort_plan(nsort.KIND_PAIRS, m)
+    fn = lambda: nsort.nsort_pairs(kt, vt, kout, vout, m, nsort.F32, tmp, tmp.numel())
+    ms = time_sort(nsort, torch, fn)
+    passes, moved = moved_bytes(traced(nsort, torch, fn), 3, m, 4, 4, plan)
     out["pairs_f32_normal_specials_2e27"] = {
         "ms": ms, "gpairs_s": m / ms / 1e6, "passes": passes,
-        "hbm_roofline_frac": passes * 16 * m / (ms / 1e3) / 1e9 / load_peaks()["hbm_gbs"]}
+        "hbm_roofline_frac": moved / (ms / 1e3) / 1e9 / load_peaks()["hbm_gbs"]}
     del vt, vout, tmp
     torch.cuda.empty_cache()
     # the same keys with 64-bit payloads (nsort_pairs64): 24 B per pair per pass
     vt = torch.arange(m, dtype=torch.int64, device="cuda")
     vout = torch.empty_like(vt)
     tmp = nsort.scratch(nsort.KIND_PAIRS64, m)
-    ms = time_sort(nsort, torch, lambda: nsort.nsort_pairs64(kt, vt, kout, vout, m, nsort.F32, tmp,
-                                                             tmp.numel()))
+    fn = lambda: nsort.nsort_pairs64(kt, vt, kout, vout, m, nsort.F32, tmp, tmp.numel())
+    ms = time_sort(nsort, torch, fn)
+    passes, moved = moved_bytes(traced(nsort, torch, fn), 3, m, 4, 8, plan)
     out["pairs64_f32_normal_specials_2e27"] = {
         "ms": ms, "gpairs_s": m / ms / 1e6, "passes": passes,
-        "hbm_roofline_frac": passes * 24 * m / (ms / 1e3) / 1e9 / load_peaks()["hbm_gbs"]}
+        "hbm_roofline_frac": moved / (ms / 1e3) / 1e9 / load_peaks()["hbm_gbs"]}
     del kt, vt, kout, vout, tmp
     torch.cuda.empty_cache()
     out.update(bench_keys64(nsort, torch))
@@ -528,14 +551,14 @@ def bench_configs(nsort, torch):
 
 def bench_keys64(nsort, torch):
     """64-bit keys (the wider-key variant): 2^27 uint64 / int64 / float64 keys
-    (1 GiB), 16 B per key per pass; the merge pass's own roofline from its
-    traced launches."""
+    (1 GiB), 16 B per key per pass; a pass's own roofline from its traced
+    launches."""
     from paper_2409_03970_gb300 import inputs
     m = 1 << 27
     peak = load_peaks()["hbm_gbs"]
     tmp = nsort.scratch(nsort.KIND_KEYS, m, dtype=nsort.U64)
     ko = torch.empty(m, dtype=torch.int64, device="cuda")
-    passes, _, _ = nsort.nsort_plan(nsort.KIND_KEYS, m, nsort.U64)
+    plan, _, _ = nsort.nsort_plan(nsort.KIND_KEYS, m, nsort.U64)
     codes = {"u64": nsort.U64, "i64": nsort.I64, "f64": nsort.F64}
     out = {}
     for dt, dist in (("u64", "uniform"), ("i64", "uniform"), ("f64", "uniform"),
@@ -544,20 +567,20 @@ def bench_keys64(nsort, torch):
         code = codes[dt]
         fn = lambda: nsort.nsort_keys(x, ko, m, code, tmp, tmp.numel())
         ms = time_sort(nsort, torch, fn)
-        nsort.nsort_trace_enable(True)            # launch durations from a traced repeat
-        time_sort(nsort, torch, fn, reps=3, warm=0)
-        tr = nsort.nsort_trace_read()
-        nsort.nsort_trace_enable(False)
+        tr = traced(nsort, torch, fn)             # launch durations from a traced repeat
+        passes, moved = moved_bytes(tr, 3, m, 8, 0, plan)
         r = {"ms": ms, "gkeys_s": m / ms / 1e6, "passes": passes,
-             "hbm_roofline_frac": passes * 16 * m / (ms / 1e3) / 1e9 / peak}
-        mk = tr.get("merge_keys64")
-        if mk and mk["launches"]:
-            lms = mk["total_ms"] / mk["launches"]
-            r["merge_keys64_ms"] = lms
-            r["merge_keys64_frac"] = 16 * m / (lms / 1e3) / 1e9 / peak
-        ts = tr.get("tile_sort_keys64")
-        if ts and ts["launches"]:
-            r["tile_sort_keys64_ms"] = ts["total_ms"] / ts["launches"]
+             "hbm_roofline_frac": moved / (ms / 1e3) / 1e9 / peak}
+        for name in ("radix_pass", "merge_keys64"):
+            k = tr.get(name)
+            if k and k["launches"]:
+                lms = k["total_ms"] / k["launches"]
+                r[f"{name}_ms"] = lms
+                r[f"{name}_frac"] = 16 * m / (lms / 1e3) / 1e9 / peak
+        for name in ("radix_histogram", "tile_sort_keys64"):
+            k = tr.get(name)
+            if k and k["launches"]:
+                r[f"{name}_ms"] = k["total_ms"] / k["launches"]
         out[f"keys_{dt}_{dist}_2e27"] = r
         del x
     del tmp, ko
@@ -568,9 +591,8 @@ def bench_keys64(nsort, torch):
 # ---- batched (segmented) and served measurements -----------------------------
 
 def bench_merge_ways(nsort, torch):
-    """Plain sorts of uniform u32 keys with one merge level per pass over
-    the array (two-way passes, the default) and with two (four-way passes):
-    ms per sort at 2^20 to 2^28."""
+    """Plain sorts of uniform u32 keys by default (digit passes) and by merge
+    passes of two levels each (four-way passes): ms per sort at 2^20 to 2^28."""
     from paper_2409_03970_gb300 import inputs
     res = {}
     for log2n in (20, 22, 24, 26, 28):
@@ -578,11 +600,11 @@ def bench_merge_ways(nsort, torch):
         x = torch.from_numpy(inputs.keys(n, "u32", "uniform", seed=0).view(np.int32)).cuda()
         y = torch.empty_like(x)
         row = {}
-        for ways, setting in ((2, nsort.FOUR_WAY_NEVER), (4, 0)):
+        for way, setting in (("default", nsort.FOUR_WAY_NEVER), ("4-way", 0)):
             prev = nsort.nsort_testing_set_four_way_min(setting)
             try:
                 tmp = nsort.scratch(nsort.KIND_KEYS, n)
-                row[f"{ways}-way_ms"] = time_sort(
+                row[f"{way}_ms"] = time_sort(
                     nsort, torch, lambda: nsort.nsort_keys(x, y, n, nsort.U32, tmp, tmp.numel()),
                     reps=11, warm=3)
                 del tmp
@@ -988,8 +1010,7 @@ def main():
     x = host_in.cuda()
     out = torch.empty_like(x)
     tmp = nsort.scratch(nsort.KIND_KEYS, n, dtype=code)
-    passes, sort_tile, merge_tile = nsort.nsort_plan(nsort.KIND_KEYS, n, code)
-    mk_name = "merge_keys64" if wide else ("merge4_keys" if args.merge_ways == 4 else "merge_keys")
+    plan_passes, sort_tile, merge_tile = nsort.nsort_plan(nsort.KIND_KEYS, n, code)
     stream = torch.cuda.current_stream()
     sh = stream.cuda_stream
 
@@ -1037,7 +1058,11 @@ def main():
     nsort.nsort_trace_enable(False)
 
     peaks = load_peaks()
-    alg_bytes_sort = passes * 2 * esize * n              # every pass reads and writes each key
+    # every pass reads and writes each key; digit passes follow one read of them
+    passes, alg_bytes_sort = moved_bytes(trace, args.steps, n, esize, 0, plan_passes)
+    by_digit = "radix_pass" in trace
+    mk_name = ("radix_pass" if by_digit else "merge_keys64" if wide else
+               "merge4_keys" if args.merge_ways == 4 else "merge_keys")
     sort_frac = alg_bytes_sort / (ms / 1e3) / 1e9 / peaks["hbm_gbs"]
     mk = trace.get(mk_name)
     roofline = None
@@ -1058,7 +1083,9 @@ def main():
                     "share_of_step": mk["total_ms"] / (traced_ms * args.steps),
                     "timing": "launch durations from a traced repeat of the timed steps "
                               f"({traced_ms:.3f} ms per traced step)"}
-    launches = sum(v["launches"] for v in trace.values()) // args.steps
+    launches = sum(v["launches"] for v in trace.values())
+    # (the histograms' trace scope holds two kernels: one clears the counters)
+    launches = (launches + trace.get("radix_histogram", {"launches": 0})["launches"]) // args.steps
 
     e2e = None
     if not args.no_e2e:
@@ -1090,13 +1117,16 @@ def main():
             "dtype": args.dtype, "data": "synthetic",
             "config": {"workload": f"plain sort, 2^{args.log2n} {args.dtype} keys, uniform, "
                                    f"seed = rank; replicas (one array per GPU)",
-                       "n": n, "passes": passes, "sort_tile": sort_tile, "merge_tile": merge_tile,
+                       "n": n, "passes": passes,
+                       "way": "digit passes" if by_digit else
+                              f"tiles of {sort_tile}, merge passes in tiles of {merge_tile}",
                        "l2": (f"inputs ({esize * n / 2**30:.2f} GiB) larger than L2; no flush"
                               if esize * n > (256 << 20) else
                               "inputs not larger than L2: a small-case run, not a bench value"),
                        "sort_hbm_roofline_frac": sort_frac,
                        "sort_algorithmic_bytes": alg_bytes_sort,
-                       "merge_levels_per_pass": 2 if args.merge_ways == 4 and not wide else 1,
+                       "merge_levels_per_pass": (0 if by_digit else
+                                                 2 if args.merge_ways == 4 and not wide else 1),
                        "parallelism": f"replicas x{world}"},
             "roofline": roofline,
             "cpu_baseline": cpu,

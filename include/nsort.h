@@ -157,9 +157,10 @@ int nsort_pairs64(const void *d_keys_in, const uint64_t *d_vals_in, void *d_keys
  * keys only).  The batch runs as three small set-up kernels (binning by
  * length on the device) and one persistent kernel that takes segments from
  * a work queue: one thread per segment of at most `tiny_width` keys, one
- * warp per segment of at most 32 x `small_ipt`, one CTA per segment of at
- * most 16 x block_threads keys, and tile sorts (32 keys per thread for keys
- * only, 16 with values) plus merge levels for longer ones.  Every
+ * warp per segment of at most 32 x `small_ipt`, as many warps as it fills
+ * (keys only; with values one CTA) per segment of at most 16 x block_threads
+ * keys, and tile sorts (32 keys per thread for keys only, 16 with values) plus
+ * merge levels for longer ones.  Every
  * step is stream-ordered with no host synchronisation, so the call can be
  * captured into a CUDA graph.  Scratch:
  * nsort_temp_bytes(NSORT_KIND_SEGMENTED[_PAIRS], n, nseg, dtype), 256-byte
