@@ -42,8 +42,8 @@ namespace serve {
 
 constexpr size_t MAX_BATCH = 4096;                 // requests per co-batch
 constexpr uint64_t MAX_BATCH_KEYS = uint64_t(1) << 24;
-// Requests of at least this many keys run one at a time (their sorts'
-// persistent merge grids fill every SM); smaller ones may pass them.
+// Requests of at least this many keys run one at a time (their sorts' passes
+// fill every SM); smaller ones may pass them.
 constexpr uint64_t LARGE_MIN_KEYS = uint64_t(1) << 22;
 
 struct BatchItem {

@@ -93,8 +93,8 @@ struct Pending {
 // requests and max_batch_keys keys.  Returns the queue positions of the
 // requests to run together (empty when nothing may start); the caller
 // removes them with take() once it has found memory for them.  Larger
-// requests run alone.  A large sort fills the GPU by itself (its persistent
-// merge grids take every SM), so two at once only share it and both finish
+// requests run alone.  A large sort fills the GPU by itself (its passes
+// take every SM), so two at once only share it and both finish
 // late; one at a time, the first finishes at its own speed.
 inline std::vector<size_t> pick_batch(const std::deque<Pending> &queue, uint64_t batch_max_keys,
                                       size_t max_batch, uint64_t max_batch_keys,
