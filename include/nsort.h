@@ -154,7 +154,7 @@ int nsort_pairs64(const void *d_keys_in, const uint64_t *d_vals_in, void *d_keys
  * d_offsets[nseg] == n (the total key count).  Empty segments are allowed.
  * Each segment is sorted on its own as nsort_keys / nsort_pairs would sort
  * it (stable when values are given; d_vals_in and d_vals_out both NULL for
- * keys only).  The batch runs as three small set-up kernels (binning by
+ * keys only).  The batch runs as four small set-up kernels (binning by
  * length on the device) and one persistent kernel that takes segments from
  * a work queue: one thread per segment of at most `tiny_width` keys, one
  * warp per segment of at most 32 x `small_ipt`, as many warps as it fills

@@ -101,32 +101,72 @@ __device__ __forceinline__ int *medium_entry(const Params &p, int c, unsigned lo
 
 // ---- set-up kernels ----------------------------------------------------------
 
-__global__ void seg_classify_kernel(Params p) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= p.nseg) return;
-  const int64_t o0 = p.off[s], o1 = p.off[s + 1];
-  const bool bad = o0 < 0 || o1 < o0 || o1 > p.n || (s == 0 && o0 != 0) ||
-                   (s == p.nseg - 1 && o1 != p.n);
-  if (bad) {
-    atomicExch(&p.ctrl->status, (int)NSORT_EINVAL);
-    return;
-  }
-  const int64_t L = o1 - o0;
+// Clears the control block (a kernel and not a memset: it can be launched
+// before its predecessors end, as in the digit sorts).
+__global__ void seg_init_kernel(Ctrl *c) {
+  static_assert(sizeof(Ctrl) % sizeof(unsigned long long) == 0, "whole words");
+  pdl_wait();
+  unsigned long long *w = reinterpret_cast<unsigned long long *>(c);
+  for (unsigned i = threadIdx.x; i < sizeof(Ctrl) / sizeof(*w); i += blockDim.x) w[i] = 0;
+}
+
+// Bins the segments by length (the lists' order is of no matter).  A CTA adds up
+// its own segments in shared memory and takes its places with one atomic add a
+// list: an add a segment, all to a few addresses, took 16.9 us for 100,000 of
+// them.  us in all, with the clearing kernel, before / now: 100,000 segments of
+// up to 1000 keys 224 / 212, of up to 65,536 5463 / 5446; 100 of up to 64 16.2 /
+// 14.2.
+constexpr int BIN_NT = 256;
+__global__ void __launch_bounds__(BIN_NT) seg_classify_kernel(Params p) {
+  constexpr int LISTS = 2 + CLASSES;   // tiny, small, medium classes
+  __shared__ unsigned count[LISTS];
+  __shared__ unsigned long long base[LISTS];
+  __shared__ unsigned long long tiles[MAXLV + 1], tile_base[MAXLV + 1];
+  const int tid = threadIdx.x;
+  if (tid < LISTS) count[tid] = 0;
+  if (tid <= MAXLV) tiles[tid] = 0;
+  __syncthreads();
+  pdl_wait();      // the previous kernel of the stream has finished writing
   Ctrl *c = p.ctrl;
-  if (L == 0) return;
-  if (L <= p.tiny_w) {
-    p.tiny_list[atomicAdd(&c->n_tiny, 1ull)] = (int)s;
-  } else if (L <= 32 * p.small_ipt) {
-    p.small_list[atomicAdd(&c->n_small, 1ull)] = (int)s;
-  } else if (L <= p.mt) {
-    int k = 0;
-    if (!p.vin)
-      while ((1024 << k) < L) ++k;   // (L <= 8192)
-    *medium_entry(p, k, atomicAdd(&c->n_medium[k], 1ull)) = (int)s;
-  } else {
-    const int64_t T = (L + p.tile - 1) / p.tile;
-    p.slot_base[s] = (int64_t)atomicAdd(&c->bucket_tiles[ceil_log2(T)], (unsigned long long)T);
+  const int64_t s = (int64_t)blockIdx.x * BIN_NT + tid;
+  int list = -1, bucket = -1;
+  unsigned at = 0;                    // place among the CTA's entries of the list
+  unsigned long long slot = 0;        // or first slot among the CTA's of the bucket
+  if (s < p.nseg) {
+    const int64_t o0 = p.off[s], o1 = p.off[s + 1];
+    const bool bad = o0 < 0 || o1 < o0 || o1 > p.n || (s == 0 && o0 != 0) ||
+                     (s == p.nseg - 1 && o1 != p.n);
+    const int64_t L = bad ? 0 : o1 - o0;
+    if (bad) {
+      atomicExch(&c->status, (int)NSORT_EINVAL);
+    } else if (L > p.mt) {
+      const int64_t T = (L + p.tile - 1) / p.tile;
+      bucket = ceil_log2(T);
+      slot = atomicAdd(&tiles[bucket], (unsigned long long)T);
+    } else if (L > 0) {
+      if (L <= p.tiny_w) {
+        list = 0;
+      } else if (L <= 32 * p.small_ipt) {
+        list = 1;
+      } else {
+        list = 2;
+        if (!p.vin)
+          while ((1024 << (list - 2)) < L) ++list;   // (L <= 8192)
+      }
+      at = atomicAdd(&count[list], 1u);
+    }
   }
+  __syncthreads();
+  if (tid < LISTS && count[tid]) {
+    unsigned long long *n = tid == 0 ? &c->n_tiny : tid == 1 ? &c->n_small : &c->n_medium[tid - 2];
+    base[tid] = atomicAdd(n, (unsigned long long)count[tid]);
+  }
+  if (tid <= MAXLV && tiles[tid]) tile_base[tid] = atomicAdd(&c->bucket_tiles[tid], tiles[tid]);
+  __syncthreads();
+  if (bucket >= 0) p.slot_base[s] = (int64_t)(tile_base[bucket] + slot);
+  if (list == 0) p.tiny_list[base[0] + at] = (int)s;
+  if (list == 1) p.small_list[base[1] + at] = (int)s;
+  if (list >= 2) *medium_entry(p, list - 2, base[list] + at) = (int)s;
 }
 
 // Lays out the work queue (one warp).
@@ -666,16 +706,13 @@ int segmented_impl(const void *d_keys_in, void *d_keys_out, const uint32_t *d_va
   p.tiny_w = cfg.tiny_width;
   p.small_ipt = cfg.small_ipt;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(p.ctrl, 0, sizeof(seg::Ctrl), st) != cudaSuccess) {
-    set_last_error(std::string("nsort_segmented: ") + cudaGetErrorString(cudaGetLastError()));
-    return NSORT_ECUDA;
-  }
-  const unsigned cblocks = (unsigned)((nseg + 255) / 256);
+  const unsigned cblocks = (unsigned)((nseg + seg::BIN_NT - 1) / seg::BIN_NT);
   {
     TraceScope tr(TK_SEG_BIN, st);
-    seg::seg_classify_kernel<<<cblocks, 256, 0, st>>>(p);
+    launch_pdl(seg::seg_init_kernel, 1, 128, 0, st, p.ctrl);
+    launch_pdl(seg::seg_classify_kernel, cblocks, seg::BIN_NT, 0, st, p);
     launch_pdl(seg::seg_plan_kernel, 1, 32, 0, st, p);
-    launch_pdl(seg::seg_owner_kernel, cblocks, 256, 0, st, p);
+    launch_pdl(seg::seg_owner_kernel, cblocks, seg::BIN_NT, 0, st, p);
   }
   int rc;
   const int per_sm = cfg.blocks_per_sm;

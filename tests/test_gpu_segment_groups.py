@@ -61,3 +61,37 @@ def test_group_edges(ns, dt, dist, copies, pairs, threads):
         else:
             wk = oracle.sort_keys(keys[a:b], dt)
         np.testing.assert_array_equal(got[a:b], wk, err_msg=f"{b - a}")
+
+
+@pytest.mark.parametrize("pairs", [False, True], ids=["keys", "pairs"])
+@pytest.mark.parametrize("nseg", [1, 255, 256, 257, 513, 1300])
+def test_binning(ns, nseg, pairs):
+    """Segments of every bin in each CTA of the binning and at its edges; calls
+    that follow one another in one scratch, the first of malformed offsets."""
+    lens = np.array([0, 1, 16, 17, 256, 257, 1024, 1025, 2048, 4096, 8192, 8193, 16385, 40000])
+    lens = lens[inputs.counter_u32(nseg, 1, 0, nseg) % lens.size]
+    lens[-1] = 33000
+    off = np.zeros(nseg + 1, np.int64)
+    np.cumsum(lens, out=off[1:])
+    n = int(off[-1])
+    bad = off.copy()
+    bad[-1] = n - 1
+    keys = inputs.keys(n, "u32", "uniform", seed=n) >> np.uint32(20)
+    k = torch.from_numpy(keys.view(np.int32)).cuda()
+    v = torch.arange(n, dtype=torch.int32, device="cuda") if pairs else None
+    ko, vo = torch.empty_like(k), torch.empty_like(v) if pairs else None
+    kind = ns.KIND_SEGMENTED_PAIRS if pairs else ns.KIND_SEGMENTED
+    tmp = torch.full((ns.nsort_temp_bytes(kind, n, nseg),), 0x5A, dtype=torch.uint8, device="cuda")
+    for offsets in (bad, off, off):
+        o = torch.from_numpy(offsets).cuda()
+        assert ns.nsort_segmented(k, ko, v, vo, o, nseg, n, 0, tmp, tmp.numel()) == ns.OK
+    assert ns.nsort_device_status(tmp) == ns.OK
+    got = ko.cpu().numpy().view(np.uint32)
+    got_v = vo.cpu().numpy().view(np.uint32) if pairs else None
+    for a, b in zip(off[:-1], off[1:]):
+        if pairs:
+            wk, wv = oracle.sort_pairs(keys[a:b], np.arange(a, b, dtype=np.uint32), "u32")
+            np.testing.assert_array_equal(got_v[a:b], wv)
+        else:
+            wk = oracle.sort_keys(keys[a:b], "u32")
+        np.testing.assert_array_equal(got[a:b], wk)
