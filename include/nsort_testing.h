@@ -1,7 +1,7 @@
 /*
- * Test hooks of libnsort: the pure host-side policy of the sort server,
- * exposed so that it can be checked on a machine without a GPU.  They make
- * no CUDA call.  Paper: none (serving is this library's extension).
+ * Test hooks of libnsort: host-side rules that can be checked on a machine
+ * without a GPU (they make no CUDA call), and self-tests of the kernels'
+ * bounded waits.  Paper: none (serving is this library's extension).
  */
 #ifndef NSORT_TESTING_H
 #define NSORT_TESTING_H
@@ -51,6 +51,11 @@ int nsort_selftest_wait(void *d_tmp, size_t tmp_bytes, uint32_t limit_us, void *
  * change.  Makes no CUDA call.  Paper: none (a merge pass of this library
  * merges one or two of the paper's merge levels). */
 uint64_t nsort_testing_set_four_way_min(uint64_t min_keys);
+
+/* The digit sorts' rule on padding: whether the `keys` positions of a tile
+ * from `first` on hold keys only or padding only, in a tile of `count` keys,
+ * so that they may be ranked in any order.  Makes no CUDA call. */
+int nsort_testing_unmixed_chunk(uint32_t first, uint32_t keys, uint32_t count);
 
 #ifdef __cplusplus
 }

@@ -27,6 +27,7 @@
 #include <type_traits>
 
 #include "nsort.h"
+#include "nsort_testing.h"
 #include "launch.h"
 #include "nsort_internal.h"
 #include "sort_device.cuh"
@@ -173,6 +174,14 @@ constexpr size_t tile_smem() {
 // positions, which would all start on one bank.
 __device__ __forceinline__ uint32_t staged(uint32_t e) { return e + (e >> 9); }
 
+// Whether the `keys` positions of a tile from `first` on hold keys only or
+// padding only, in a tile of `count` keys: else its padding, which has the
+// largest digit throughout, has to be ranked behind its keys of that digit,
+// and the order in which the lanes of one atomic are served is not specified.
+__host__ __device__ constexpr bool unmixed_chunk(uint32_t first, uint32_t keys, uint32_t count) {
+  return first + keys <= count || first >= count;
+}
+
 // One tile's share of one digit pass, by one CTA: IPT keys per thread,
 // TILE = 512 IPT in all, in chunks of 16 IPT: the first halves of the warps
 // take the first 16 chunks, the second halves the others, lane l of a
@@ -191,7 +200,7 @@ __device__ __forceinline__ uint32_t staged(uint32_t e) { return e + (e >> 9); }
 //
 // Ranking where order is free.  Keys without payloads need to stay in order
 // only if they differ in the lower digits, by which the array is sorted
-// already.  A tile whose first and last keys agree in them (every tile of
+// already.  A full tile whose first and last keys agree in them (every one of
 // the first pass, nearly every one of the second) is ranked in any order:
 // one counter per digit and lane, so that no two lanes of a warp meet on an
 // address or a bank, and one atomic per key.
@@ -408,10 +417,12 @@ struct DigitTile {
       for (int i = I0; i < I1; ++i)
         stage[staged(atomicAdd(mine + COPIES * digit(r[i]), 1u))] = r[i];
     } else {
-      // the keys of this warp may be order-free even if the tile's are not
+      // The keys of this warp may be order-free even if the tile's are not,
+      // but never beside padding (unmixed_chunk).
       const K f = __shfl_sync(0xffffffffu, r[0], lane & 16) & low;
       const K l = __shfl_sync(0xffffffffu, r[IPT - 1], lane | 15) & low;
-      if (__all_sync(0xffffffffu, f == l)) {
+      const bool unmixed = unmixed_chunk(e0 - (lane & 15), 16 * IPT, count);
+      if (__all_sync(0xffffffffu, f == l && unmixed)) {
 #pragma unroll
         for (int i = I0; i < I1; ++i)
           stage[staged(atomicAdd(mine + 2 * digit(r[i]), 1u << 16) >> 16)] = r[i];
@@ -1106,6 +1117,10 @@ int radix_sort_typed(const Plan &p, bool *sorted, const K *in, const V *vin, K *
 }
 
 }  // namespace
+
+extern "C" int nsort_testing_unmixed_chunk(uint32_t first, uint32_t keys, uint32_t count) {
+  return unmixed_chunk(first, keys, count);
+}
 
 int radix_sort_keys(const Plan &p, bool *sorted, const uint32_t *in, uint32_t *out, int dt,
                     void *tmp, cudaStream_t st) {
