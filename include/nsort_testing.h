@@ -52,11 +52,6 @@ int nsort_selftest_wait(void *d_tmp, size_t tmp_bytes, uint32_t limit_us, void *
  * merges one or two of the paper's merge levels). */
 uint64_t nsort_testing_set_four_way_min(uint64_t min_keys);
 
-/* The digit sorts' rule on padding: whether the `keys` positions of a tile
- * from `first` on hold keys only or padding only, in a tile of `count` keys,
- * so that they may be ranked in any order.  Makes no CUDA call. */
-int nsort_testing_unmixed_chunk(uint32_t first, uint32_t keys, uint32_t count);
-
 #ifdef __cplusplus
 }
 #endif

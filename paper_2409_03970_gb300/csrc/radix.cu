@@ -27,7 +27,6 @@
 #include <type_traits>
 
 #include "nsort.h"
-#include "nsort_testing.h"
 #include "launch.h"
 #include "nsort_internal.h"
 #include "sort_device.cuh"
@@ -173,14 +172,6 @@ constexpr size_t tile_smem() {
 // free order a tile of one digit gives every lane its own 512 consecutive
 // positions, which would all start on one bank.
 __device__ __forceinline__ uint32_t staged(uint32_t e) { return e + (e >> 9); }
-
-// Whether the `keys` positions of a tile from `first` on hold keys only or
-// padding only, in a tile of `count` keys: else its padding, which has the
-// largest digit throughout, has to be ranked behind its keys of that digit,
-// and the order in which the lanes of one atomic are served is not specified.
-__host__ __device__ constexpr bool unmixed_chunk(uint32_t first, uint32_t keys, uint32_t count) {
-  return first + keys <= count || first >= count;
-}
 
 // One tile's share of one digit pass, by one CTA: IPT keys per thread,
 // TILE = 512 IPT in all, in chunks of 16 IPT: the first halves of the warps
@@ -417,15 +408,26 @@ struct DigitTile {
       for (int i = I0; i < I1; ++i)
         stage[staged(atomicAdd(mine + COPIES * digit(r[i]), 1u))] = r[i];
     } else {
-      // The keys of this warp may be order-free even if the tile's are not,
-      // but never beside padding (unmixed_chunk).
+      // the keys of this warp may be order-free even if the tile's are not
       const K f = __shfl_sync(0xffffffffu, r[0], lane & 16) & low;
       const K l = __shfl_sync(0xffffffffu, r[IPT - 1], lane | 15) & low;
-      const bool unmixed = unmixed_chunk(e0 - (lane & 15), 16 * IPT, count);
-      if (__all_sync(0xffffffffu, f == l && unmixed)) {
+      if (__all_sync(0xffffffffu, f == l)) {
+        if (count == TILE) {
 #pragma unroll
-        for (int i = I0; i < I1; ++i)
-          stage[staged(atomicAdd(mine + 2 * digit(r[i]), 1u << 16) >> 16)] = r[i];
+          for (int i = I0; i < I1; ++i)
+            stage[staged(atomicAdd(mine + 2 * digit(r[i]), 1u << 16) >> 16)] = r[i];
+        } else {
+          // Padding takes no part.  It has the largest digit throughout, and
+          // the lanes of one atomic are served in no specified order, so that
+          // it could take the place of a key; its own places, all from `count`
+          // on, stay empty.  (Ranked with the keys, all of it on one counter,
+          // it also took longer: 4.0e6 u32 keys 83.3 -> 78.3 us, 1.2e6 int64
+          // 87.9 -> 83.4.)
+#pragma unroll
+          for (int i = I0; i < I1; ++i)
+            if (e0 + 16 * i < count)
+              stage[staged(atomicAdd(mine + 2 * digit(r[i]), 1u << 16) >> 16)] = r[i];
+        }
       } else {
 #pragma unroll
         for (int i = I0; i < I1; ++i) stage[staged(rank_stable(mine, r[i]))] = r[i];
@@ -1117,10 +1119,6 @@ int radix_sort_typed(const Plan &p, bool *sorted, const K *in, const V *vin, K *
 }
 
 }  // namespace
-
-extern "C" int nsort_testing_unmixed_chunk(uint32_t first, uint32_t keys, uint32_t count) {
-  return unmixed_chunk(first, keys, count);
-}
 
 int radix_sort_keys(const Plan &p, bool *sorted, const uint32_t *in, uint32_t *out, int dt,
                     void *tmp, cudaStream_t st) {

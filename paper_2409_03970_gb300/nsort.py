@@ -128,8 +128,6 @@ def _load():
         lib.nsort_selftest_wait.restype = i32
         lib.nsort_testing_set_four_way_min.argtypes = [u64]
         lib.nsort_testing_set_four_way_min.restype = u64
-        lib.nsort_testing_unmixed_chunk.argtypes = [ctypes.c_uint32] * 3
-        lib.nsort_testing_unmixed_chunk.restype = i32
         lib.nsort_keys_noalloc.argtypes = [vp, vp, u64, i32, vp]
         lib.nsort_keys_noalloc.restype = i32
         lib.nsort_keys_noalloc_status.argtypes = [vp]
@@ -396,12 +394,6 @@ def nsort_testing_set_four_way_min(min_keys: int) -> int:
     """Smallest 32-bit key sort that merges two levels per pass (test hook);
     returns the previous setting."""
     return int(_load().nsort_testing_set_four_way_min(min_keys))
-
-
-def nsort_testing_unmixed_chunk(first: int, keys: int, count: int) -> bool:
-    """Whether positions first .. first + keys - 1 of a tile of `count` keys
-    hold keys only or padding only (test hook)."""
-    return bool(_load().nsort_testing_unmixed_chunk(first, keys, count))
 
 
 FOUR_WAY_NEVER = (1 << 64) - 1

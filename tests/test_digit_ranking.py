@@ -3,39 +3,51 @@ DigitTile::rank): half-warps take chunks of 16 x IPT keys, 16 at a time, and ran
 a chunk whose sorted digits agree with one atomic per key.  The order in which
 the lanes of one atomic are served is not specified, so the model serves them
 from either end: whatever the order, the staged keys below `count` have to be
-the tile's keys and none of its padding.  Which chunks may be ranked so is the
-library's own rule (nsort_testing_unmixed_chunk)."""
+the tile's keys and none of its padding.  Who takes part in those atomics is
+read from the source."""
+import os
+import re
+
 import numpy as np
 import pytest
 
-import __graft_entry__
-from paper_2409_03970_gb300 import nsort
-
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 HALF_WARPS = 32
 PAD = 0xFFFFFFFF
 
 
-@pytest.fixture(scope="module", autouse=True)
-def built():
-    __graft_entry__.build()
+def padding_takes_part():
+    """Whether a free-order atomic of a partial tile is done for padding too."""
+    with open(os.path.join(ROOT, "paper_2409_03970_gb300", "csrc", "radix.cu")) as f:
+        text = re.sub(r"//[^\n]*|#pragma[^\n]*", "", f.read())
+    branch = re.search(r"if \(__all_sync\(0xffffffffu, f == l\)\) \{(.*?)\n      \} else \{", text,
+                       re.S).group(1)
+    full, _, partial = branch.partition("} else {")
+    return not (re.match(r"\s*if \(count == TILE\) \{", full) and
+                re.search(r"if \(e0 \+ 16 \* i < count\)\s*stage\[", partial))
 
 
 def stage(keys, count, ipt, shift, descending):
-    """The tile's keys in the order of one pass, all chunks whose sorted digits
-    agree and that the rule allows ranked with lanes served in the given order."""
+    """The tile's keys in the order of one pass, every chunk whose sorted digits
+    agree ranked with the lanes served in the given order; PAD where nothing
+    is staged."""
     low = (1 << shift) - 1
     digit = (keys >> shift) & 0xFF
     chunk = 16 * ipt
-    staged = np.zeros_like(keys)
-    at = np.concatenate([[0], np.cumsum(np.bincount(digit, minlength=256))[:-1]])
+    staged = np.full_like(keys, PAD)
+    counts = np.stack([np.bincount(digit[c * chunk:(c + 1) * chunk], minlength=256)
+                       for c in range(HALF_WARPS)])
+    start = np.concatenate([[0], np.cumsum(counts.sum(0))[:-1]])   # the digit's place in the tile
+    pads = padding_takes_part()
     for c in range(HALF_WARPS):
+        at = start + counts[:c].sum(0)                             # this half-warp's counters
         first = c * chunk
-        free = ((keys[first] ^ keys[first + chunk - 1]) & low) == 0 and \
-            nsort.nsort_testing_unmixed_chunk(first, chunk, count)
+        free = ((keys[first] ^ keys[first + chunk - 1]) & low) == 0
         for i in range(ipt):
-            lanes = range(15, -1, -1) if free and descending else range(16)
-            for lane in lanes:
+            for lane in range(15, -1, -1) if free and descending else range(16):
                 e = first + 16 * i + lane
+                if free and not pads and e >= count:
+                    continue
                 staged[at[digit[e]]] = keys[e]
                 at[digit[e]] += 1
     return staged
@@ -57,10 +69,3 @@ def test_no_key_lost_to_padding(ipt, descending):
                 np.testing.assert_array_equal(np.sort(x[:count]), np.sort(keys[:count]))
                 x[count:] = PAD
             np.testing.assert_array_equal(x[:count], np.sort(keys[:count]))
-
-
-def test_rule():
-    assert nsort.nsort_testing_unmixed_chunk(64, 64, 128)       # ends with the keys
-    assert nsort.nsort_testing_unmixed_chunk(128, 64, 128)      # begins behind them
-    assert not nsort.nsort_testing_unmixed_chunk(64, 64, 127)
-    assert not nsort.nsort_testing_unmixed_chunk(64, 64, 65)
