@@ -148,6 +148,28 @@ __device__ __forceinline__ void store_relaxed(uint32_t *p, uint32_t v) {
   asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// Who writes what a kernel reads: no one in the kernel's life (the read-only
+// path); the kernel before it, which may still be writing when this one starts
+// (plain loads, not moved over the wait for it; ld.global.cg there costs 2-4%
+// of a wave sort); or this kernel's other CTAs (loads from L2).
+enum Writer { NOBODY, PREDECESSOR, THIS_KERNEL };
+template <Writer W>
+__device__ __forceinline__ uint32_t load_from(const uint32_t *p) {
+  if constexpr (W == NOBODY) return __ldg(p);
+  if constexpr (W == THIS_KERNEL) return __ldcg(p);
+  uint32_t v;
+  asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+template <Writer W>
+__device__ __forceinline__ uint64_t load_from(const uint64_t *p) {
+  if constexpr (W == NOBODY) return __ldg(p);
+  if constexpr (W == THIS_KERNEL) return __ldcg(p);
+  uint64_t v;
+  asm volatile("ld.global.u64 %0, [%1];" : "=l"(v) : "l"(p));
+  return v;
+}
+
 // Whether a wait that began at t0 (0: begins now) has lasted two seconds.
 __device__ __forceinline__ bool gave_up(uint64_t &t0) {
   const uint64_t now = global_ns();
@@ -252,17 +274,17 @@ struct DigitTile {
     for (int i = 0; i < COPIES * BINS / 4 / NT; ++i) c4[tid + NT * i] = make_uint4(0, 0, 0, 0);
   }
 
-  // The tile's keys from p (COHERENT: written earlier in the same launch).
-  template <bool COHERENT>
+  // The tile's keys from p.
+  template <Writer FROM>
   __device__ __forceinline__ void load(const K *p, K (&r)[IPT]) const {
     p += e0;
     if (count == TILE) {
 #pragma unroll
-      for (int i = 0; i < IPT; ++i) r[i] = COHERENT ? __ldcg(p + 16 * i) : __ldg(p + 16 * i);
+      for (int i = 0; i < IPT; ++i) r[i] = load_from<FROM>(p + 16 * i);
     } else {
 #pragma unroll
       for (int i = 0; i < IPT; ++i)
-        r[i] = e0 + 16 * i < count ? (COHERENT ? __ldcg(p + 16 * i) : __ldg(p + 16 * i)) : K(0);
+        r[i] = e0 + 16 * i < count ? load_from<FROM>(p + 16 * i) : K(0);
     }
   }
   // padding: the largest key, behind every real one
@@ -485,7 +507,7 @@ struct DigitTile {
 
   // The payloads, from p, take the keys' places in the staging buffer, as
   // many positions at a time as fit, and follow them.
-  template <bool COHERENT>
+  template <Writer FROM>
   __device__ __forceinline__ void move_values(const V *p, V *dst, uint32_t n, bool checked,
                                               const uint32_t (&pos2)[NPOS],
                                               const uint32_t (&dig4)[NDIG]) const {
@@ -506,7 +528,7 @@ struct DigitTile {
           for (int i = i0; i < i0 + VB; ++i) {
             const uint32_t pos = (pos2[i / 2] >> (16 * (i & 1))) & 0xFFFFu;
             if ((ROUNDS == 1 || (int)(pos / RT) == q) && e0 + 16 * i < count)
-              vstage[staged(pos - q * RT)] = COHERENT ? __ldcg(p + 16 * i) : __ldg(p + 16 * i);
+              vstage[staged(pos - q * RT)] = load_from<FROM>(p + 16 * i);
           }
           asm volatile("" ::: "memory");
         }
@@ -557,7 +579,10 @@ __device__ __forceinline__ uint32_t load_of_cta(const uint32_t *p, uint32_t c) {
 // over all of them, since no tile is done before the others start.  CL > 1:
 // a cluster of CL CTAs shares an entry of the counts (CL tiles in a row),
 // which leaves room in the scratch for short tiles: the CTAs exchange their
-// counts through distributed shared memory.
+// counts through distributed shared memory.  A wave pass is alive while the
+// pass before it still writes (pdl_trigger), so it reads what that one and the
+// histogram kernel write as such; a look-back pass starts when its
+// predecessor has ended, and may take the read-only path.
 //
 // What bounds it (ncu at 2^26 uniform u32 keys): the LSU data pipe in the
 // stable passes (20-22 shared-memory wavefronts for 32 keys beside the
@@ -581,10 +606,9 @@ __device__ __forceinline__ uint32_t load_of_cta(const uint32_t *p, uint32_t c) {
 constexpr uint32_t AHEAD = 76;   // tiles: a quarter of those that run at once
 template <typename K, typename V, int IPT, bool FIRST, bool LAST, bool WAVE, int CL = 1>
 __global__ void __launch_bounds__(NT, 2) radix_pass_kernel(
-    const K *__restrict__ src, const V *__restrict__ vsrc, K *__restrict__ dst,
-    V *__restrict__ vdst, uint32_t n, int shift, KeyMap<K> map_i, KeyMap<K> map_o,
-    const uint32_t *__restrict__ hist, uint32_t *state, uint32_t parity, uint32_t *ticket,
-    int *status) {
+    const K *src, const V *vsrc, K *__restrict__ dst, V *__restrict__ vdst, uint32_t n, int shift,
+    KeyMap<K> map_i, KeyMap<K> map_o, const uint32_t *hist, uint32_t *state, uint32_t parity,
+    uint32_t *ticket, int *status) {
   using T = DigitTile<K, V, IPT>;
   extern __shared__ __align__(16) unsigned char rp_smem[];
   __shared__ typename T::Shared sh;
@@ -611,7 +635,13 @@ __global__ void __launch_bounds__(NT, 2) radix_pass_kernel(
   t.count = base >= n ? 0u : (n - base < (uint32_t)T::TILE ? n - base : (uint32_t)T::TILE);
   const uint32_t count = t.count;
   K r[IPT];
-  t.template load<false>(src + base, r);
+  t.template load<WAVE ? PREDECESSOR : NOBODY>(src + base, r);
+  // (WAVE) the digit's count in the array, asked for ahead of its use: at once
+  // in the short tiles of clusters (200,003 u32 keys 28.6 -> 27.5 us), else
+  // after the counting, where it keeps a register for less long (2.3e6 int64
+  // keys 138.6 us, 141 at once)
+  [[maybe_unused]] uint32_t digit_total = 0;
+  if constexpr (WAVE && CL > 1) digit_total = load_from<PREDECESSOR>(hist + (tid >> 1));
   t.prefetch(vsrc + base);
   if constexpr (!WAVE) {   // the keys of the tile that starts when this one ends
     constexpr uint32_t LINE = 128 / sizeof(K);
@@ -643,11 +673,12 @@ __global__ void __launch_bounds__(NT, 2) radix_pass_kernel(
   if constexpr (CL == 1) publish(total);
   if (!(tid & 1)) sh.tile_total[d] = total;
   if constexpr (CL > 1) cluster_arrive();   // the count is there for the other CTAs
+  if constexpr (WAVE && CL == 1) digit_total = load_from<PREDECESSOR>(hist + d);
   const uint32_t tbase = t.sum_below(total);   // where the digit starts in the tile
   if (!(tid & 1)) sh.tile_base[d] = tbase;
   t.place_counters(tbase + (tid & 1 ? other : 0u), kept);
   [[maybe_unused]] uint32_t excl0 = 0;   // (WAVE) all smaller digits, and the cluster's lower ranks
-  if constexpr (WAVE) excl0 = t.sum_below(hist[d]);
+  if constexpr (WAVE) excl0 = t.sum_below(digit_total);
   if constexpr (CL > 1) {
     cluster_wait();
     uint32_t all = 0, lower = 0;
@@ -777,7 +808,7 @@ __global__ void __launch_bounds__(NT, 2) radix_pass_kernel(
   const bool checked = fault || count != T::TILE;
   uint32_t dig4[T::NDIG];
   t.template write_keys<LAST>(dst, n, checked, map_o, dig4);
-  t.template move_values<false>(vsrc + base, vdst, n, checked, pos2, dig4);
+  t.template move_values<WAVE ? PREDECESSOR : NOBODY>(vsrc + base, vdst, n, checked, pos2, dig4);
   if constexpr (CL > 1) cluster_wait();
 }
 
@@ -812,7 +843,7 @@ __global__ void __launch_bounds__(NT, 1) radix_cluster_kernel(
     t.set_digit(8 * dg);
     t.clear();
     K r[IPT];
-    t.template load<true>(src + base, r);
+    t.template load<THIS_KERNEL>(src + base, r);
     t.prefetch(vsrc + base);
     if (dg == 0) {
 #pragma unroll
@@ -848,7 +879,7 @@ __global__ void __launch_bounds__(NT, 1) radix_cluster_kernel(
     uint32_t dig4[T::NDIG];
     // (checked throughout: the positions come from keys that were read again)
     t.template write_keys<true>(dst, n, true, map_o, dig4);
-    t.template move_values<true>(vsrc + base, vdst, n, true, pos2, dig4);
+    t.template move_values<THIS_KERNEL>(vsrc + base, vdst, n, true, pos2, dig4);
     src = dst;
     vsrc = vdst;
     cluster_arrive();   // the pass is written, and no CTA reads another's counts any more
