@@ -43,6 +43,20 @@ int nsort_policy_arena_replay(uint64_t capacity, const int64_t *ops, int nops,
  * or faulting a GPU.  Paper: none. */
 int nsort_selftest_wait(void *d_tmp, size_t tmp_bytes, uint32_t limit_us, void *stream);
 
+/* Runs the digit passes' waits for the key counts of other tiles (which = 0:
+ * look-back passes; 1: passes whose tiles all run at once; 2: those in
+ * clusters of four) on counts that never come, with a limit of limit_us (two
+ * million at most) microseconds, in the pass kernels themselves: the second and the third
+ * tile (group of four tiles) of a pass whose first is left out, in a launch
+ * each.  Both give up and return normally.  d_tmp (at least
+ * NSORT_SELFTEST_DIGIT_BYTES, 256-byte aligned) holds their status words
+ * (NSORT_ETIMEOUT) at words 0 and 2, and from byte 256 on the pass's destination,
+ * filled with 0xA5 before: a tile that gives up writes none of its keys.  Paper:
+ * none. */
+#define NSORT_SELFTEST_DIGIT_BYTES (1u << 19)
+int nsort_selftest_digit_waits(int which, void *d_tmp, size_t tmp_bytes, uint32_t limit_us,
+                               void *stream);
+
 /* Sets the smallest key count at which a sort of 32-bit keys merges two
  * levels per pass over the array (four-way passes) and returns the previous
  * setting.  0 selects four-way passes for every sort with at least two

@@ -27,6 +27,7 @@
 #include <type_traits>
 
 #include "nsort.h"
+#include "nsort_testing.h"
 #include "launch.h"
 #include "nsort_internal.h"
 #include "sort_device.cuh"
@@ -37,6 +38,7 @@ namespace nsort {
 namespace {
 
 constexpr int BINS = 256;
+constexpr int WAIT_US = 2000000;   // limit of a pass's wait for other tiles
 
 // Sets the histograms and the tickets to zero.  A kernel and not a memset,
 // since kernels can be launched before their predecessors end: us, memset and
@@ -55,7 +57,8 @@ __global__ void radix_init_kernel(uint32_t *words, int n) {
 // group counts in its own copy of the counters (COPIES of them, copy = lane
 // mod COPIES, the copies of one counter in different banks), so that equal
 // digits of a warp do not queue up on one address.  Also sets the passes'
-// look-back words to "no entry" and the status word to NSORT_OK.
+// look-back words to "no entry", the status word to NSORT_OK and the word behind
+// it to the limit of the passes' waits.
 // SMALL: the first pass may start to wait early (and take its tickets, which
 // are zero by then: after pdl_wait).
 template <typename K, int NT, int COPIES, bool SMALL>
@@ -71,7 +74,10 @@ __global__ void __launch_bounds__(NT) radix_histogram_kernel(const K *__restrict
   const int64_t gsize = (int64_t)gridDim.x * NT;
   pdl_wait();
   for (int64_t i = gtid; i < state_words; i += gsize) state[i] = 0xFFFFFFFFu;
-  if (gtid == 0) *status = NSORT_OK;
+  if (gtid == 0) {
+    status[0] = NSORT_OK;
+    status[1] = WAIT_US;
+  }
   if (SMALL) pdl_trigger();
   __syncthreads();
   uint32_t *mine = rh_cnt + (tid & (COPIES - 1));
@@ -170,11 +176,14 @@ __device__ __forceinline__ uint64_t load_from(const uint64_t *p) {
   return v;
 }
 
-// Whether a wait that began at t0 (0: begins now) has lasted two seconds.
-__device__ __forceinline__ bool gave_up(uint64_t &t0) {
+// Whether a wait that began at t0 (0: begins now) has lasted as many
+// microseconds as the word behind the status word says.  (Read there, by a wait
+// that has to wait: as an argument of the passes it costs some of them a
+// register that they don't have.)
+__device__ __forceinline__ bool gave_up(uint64_t &t0, const int *status) {
   const uint64_t now = global_ns();
   if (!t0) t0 = now;
-  return now - t0 > 2000000000ull;
+  return now - t0 > load_relaxed(reinterpret_cast<const uint32_t *>(status) + 1) * 1000ull;
 }
 
 struct NoValue {};
@@ -730,7 +739,7 @@ __global__ void __launch_bounds__(NT, 2) radix_pass_kernel(
             acc[6] += x.w & 0xFFFFu; acc[7] += x.w >> 16;
             break;
           }
-          if (flags || gave_up(t0)) {
+          if (flags || gave_up(t0, status)) {
             flags = 2;
             break;
           }
@@ -786,7 +795,7 @@ __global__ void __launch_bounds__(NT, 2) radix_pass_kernel(
             }
           }
           p -= used * BINS;
-          if (!used && gave_up(t0)) {
+          if (!used && gave_up(t0, status)) {
             flags = 2;
             break;
           }
@@ -1149,7 +1158,58 @@ int radix_sort_typed(const Plan &p, bool *sorted, const K *in, const V *vin, K *
   return NSORT_OK;
 }
 
+// Self-test of a pass's wait for other tiles' counts: the pass's turns 1 and 2
+// in a launch each, over a scratch where turn 0 never publishes any.  tmp:
+// status words and limits of the two | destination | keys | histogram, ticket |
+// counts.
+__global__ void selftest_waits_kernel(int *status, uint32_t *ticket, int limit_us) {
+  for (int turn = 0; turn < 2; ++turn) {
+    status[2 * turn] = NSORT_OK;
+    status[2 * turn + 1] = limit_us;
+  }
+  *ticket = 1;
+}
+template <int IPT, bool WAVE, int CL>
+void selftest_waits(char *tmp, int limit_us, cudaStream_t st) {
+  constexpr size_t TURN = NT * IPT * CL, N = 3 * TURN;
+  constexpr size_t DST = 256, SRC = DST + N * 4, HIST = SRC + N * 4, TICKET = HIST + BINS * 4,
+                   STATE = TICKET + 256, END = STATE + 3 * BINS * 4;
+  static_assert(END <= NSORT_SELFTEST_DIGIT_BYTES, "fits");
+  int *status = reinterpret_cast<int *>(tmp);
+  uint32_t *ticket = reinterpret_cast<uint32_t *>(tmp + TICKET);
+  cudaMemsetAsync(tmp + DST, 0xA5, N * 4, st);
+  cudaMemsetAsync(tmp + SRC, 0, STATE - SRC, st);   // keys of one digit
+  cudaMemsetAsync(tmp + STATE, 0xFF, END - STATE, st);
+  selftest_waits_kernel<<<1, 1, 0, st>>>(status, ticket, limit_us);
+  const KeyMap<uint32_t> none = {0u, 0u};
+  const NoValue *vsrc = nullptr;
+  NoValue *vdst = nullptr;
+  for (int turn = 0; turn < 2; ++turn)
+    launch_pdl<CL>(radix_pass_kernel<uint32_t, NoValue, IPT, WAVE, WAVE, WAVE, CL>, CL, NT,
+                   tile_smem<uint32_t, IPT>(), st, reinterpret_cast<const uint32_t *>(tmp + SRC),
+                   vsrc, reinterpret_cast<uint32_t *>(tmp + DST), vdst, (uint32_t)N, 0, none, none,
+                   reinterpret_cast<const uint32_t *>(tmp + HIST),
+                   reinterpret_cast<uint32_t *>(tmp + STATE), 0u, ticket, status + 2 * turn);
+}
+
 }  // namespace
+
+extern "C" int nsort_selftest_digit_waits(int which, void *d_tmp, size_t tmp_bytes,
+                                          uint32_t limit_us, void *stream) {
+  if (which < 0 || which > 2 || limit_us > (uint32_t)WAIT_US || !d_tmp || tmp_bytes < NSORT_SELFTEST_DIGIT_BYTES ||
+      (reinterpret_cast<uintptr_t>(d_tmp) & 255))
+    return NSORT_EINVAL;
+  int sms = 0, wave_clusters = 0;
+  bool cluster = false;
+  if (radix_setup<uint32_t, NoValue>(&sms, &cluster, &wave_clusters) != NSORT_OK)
+    return radix_status(cudaGetLastError(), "radix set-up");
+  char *t = static_cast<char *>(d_tmp);
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (which == 0) selftest_waits<large_ipt<uint32_t>(), false, 1>(t, (int)limit_us, st);
+  else if (which == 1) selftest_waits<wave_ipt<uint32_t>(), true, 1>(t, (int)limit_us, st);
+  else selftest_waits<WAVE_CL_IPT, true, WAVE_CL>(t, (int)limit_us, st);
+  return radix_status(cudaSuccess, "nsort_selftest_digit_waits");
+}
 
 int radix_sort_keys(const Plan &p, bool *sorted, const uint32_t *in, uint32_t *out, int dt,
                     void *tmp, cudaStream_t st) {

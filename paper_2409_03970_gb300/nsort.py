@@ -126,6 +126,8 @@ def _load():
         lib.nsort_policy_arena_replay.restype = i32
         lib.nsort_selftest_wait.argtypes = [vp, sz, ctypes.c_uint32, vp]
         lib.nsort_selftest_wait.restype = i32
+        lib.nsort_selftest_digit_waits.argtypes = [i32, vp, sz, ctypes.c_uint32, vp]
+        lib.nsort_selftest_digit_waits.restype = i32
         lib.nsort_testing_set_four_way_min.argtypes = [u64]
         lib.nsort_testing_set_four_way_min.restype = u64
         lib.nsort_keys_noalloc.argtypes = [vp, vp, u64, i32, vp]
@@ -388,6 +390,16 @@ def nsort_selftest_wait(tmp, limit_us: int = 20000, stream=None) -> int:
     """Runs the library's bounded waits on events that never happen (test hook)."""
     return _load().nsort_selftest_wait(_ptr(tmp), tmp.numel() if hasattr(tmp, "numel") else 512,
                                        limit_us, _stream(stream))
+
+
+SELFTEST_DIGIT_BYTES = 1 << 19
+
+
+def nsort_selftest_digit_waits(which: int, tmp, limit_us: int, stream=None) -> int:
+    """Waits of the digit passes (0: look-back, 1: wave, 2: wave in clusters) on
+    counts that never come."""
+    return _load().nsort_selftest_digit_waits(which, _ptr(tmp), tmp.numel() * tmp.element_size(),
+                                              limit_us, _stream(stream))
 
 
 def nsort_testing_set_four_way_min(min_keys: int) -> int:
