@@ -130,7 +130,9 @@ __global__ void __launch_bounds__(NT) radix_histogram_kernel(const K *__restrict
 
 // Look-back word of (tile, digit): bit 31 the pass's parity, bit 30 set when
 // the count is that of every tile up to this one (and of every smaller
-// digit), else it is the tile's own, bits 29..0 the count.  A word of the
+// digit), else it is the tile's own, bits 29..0 the count.  Bits 30..0 all set: a
+// tile up to this one gave up waiting, and there is no count (2^30 - 1 as a
+// count says that no key of the digit is left in later tiles).  A word of the
 // other parity is no entry yet: the histogram kernel fills the words with
 // ones (parity 1, the pass before the first) and every pass overwrites all
 // of them.
@@ -796,16 +798,18 @@ __global__ void __launch_bounds__(NT, 2) radix_pass_kernel(
           }
           p -= used * BINS;
           if (!used && gave_up(t0, status)) {
+            excl = LB_COUNT;   // there is no sum, which later tiles have to see as well
             flags = 2;
             break;
           }
         } while (!done);
       }
       const uint32_t c = sh.tile_total[tid];
-      store_relaxed(word, parity | LB_INCL | ((excl + c) & LB_COUNT));
+      store_relaxed(word, parity | LB_INCL | min(excl + c, LB_COUNT));
       sh.gbase[tid] = excl - sh.tile_base[tid];
-      // holds for every digit unless the keys changed while they were sorted
-      if (excl + c > n + (tid == BINS - 1 ? T::TILE - count : 0)) flags |= 1;
+      // holds for every digit unless a tile before gave up, or the keys changed
+      // while they were sorted
+      if (excl + c > n + (tid == BINS - 1 ? T::TILE - count : 0)) flags |= excl >= LB_COUNT ? 2 : 1;
     }
   }
   const bool fault = __syncthreads_or(flags);

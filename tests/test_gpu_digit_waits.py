@@ -51,3 +51,12 @@ def test_waits_give_up_and_report(ns, which):
     assert ns.nsort_keys(xt, out, n, ns.F32, sc, sc.numel()) == ns.OK
     assert ns.nsort_device_status(sc) == ns.OK
     np.testing.assert_array_equal(out.cpu().numpy().view(np.uint32), oracle.sort_keys(x, "f32"))
+
+
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_later_tiles_do_not_build_on_a_wait_that_gave_up(ns, which):
+    """The tile after the one that gave up (its launch begins when that has
+    ended) gives up as well, and neither writes a key."""
+    first, second, untouched, seconds = run(ns, which, 20_000)
+    assert (first, second) == (ns.ETIMEOUT, ns.ETIMEOUT)
+    assert untouched and seconds < 5.0
