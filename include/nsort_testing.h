@@ -57,6 +57,14 @@ int nsort_selftest_wait(void *d_tmp, size_t tmp_bytes, uint32_t limit_us, void *
 int nsort_selftest_digit_waits(int which, void *d_tmp, size_t tmp_bytes, uint32_t limit_us,
                                void *stream);
 
+/* nsort_keys, nsort_pairs or nsort_pairs64 (kind; values NULL for keys) by
+ * the merge passes of the plan, which those take for arrays of 2^30 keys or
+ * more (32-bit keys) and for some sizes of 64-bit keys: the same arguments,
+ * scratch, status word and result.  n must need at least one merge pass. */
+int nsort_testing_merge_sort(int kind, const void *d_keys_in, const void *d_vals_in,
+                             void *d_keys_out, void *d_vals_out, uint64_t n, int dtype,
+                             void *d_tmp, size_t tmp_bytes, void *stream);
+
 /* Sets the smallest key count at which a sort of 32-bit keys merges two
  * levels per pass over the array (four-way passes) and returns the previous
  * setting.  0 selects four-way passes for every sort with at least two

@@ -1910,17 +1910,10 @@ static void launch_merge_staged64(const uint64_t *src, uint64_t *dst, int64_t n,
 #undef NSORT_MK64
 }
 
-int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void *tmp,
-                     cudaStream_t st) {
-  const Plan p = make_plan(NSORT_KIND_KEYS, (uint64_t)n, dt);
-  if (p.merge_passes == 0) {
-    TraceScope tr(TK_TILE_SORT_KEYS64, st);
-    small_sort_keys64(in, out, (int)n, dt, st);
-    return launch_status("small_sort_keys64");
-  }
-  bool sorted = false;
-  int rc = radix_sort_keys64(p, &sorted, in, out, dt, tmp, st);
-  if (sorted || rc != NSORT_OK) return rc;
+// The sort by the plan's merge passes (at least one).
+static int merge_sort_keys64(const Plan &p, const uint64_t *in, uint64_t *out, int dt, void *tmp,
+                             cudaStream_t st) {
+  const int64_t n = p.n;
   char *t = static_cast<char *>(tmp);
   uint64_t *bufs[2] = {out, reinterpret_cast<uint64_t *>(t + p.keys_off)};
   int64_t *split = reinterpret_cast<int64_t *>(t + p.split_off);
@@ -1935,7 +1928,7 @@ int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void 
     TraceScope tr(TK_TILE_SORT_KEYS64, st);
     launch_tile_sort_keys64(in, bufs[cur], n, dt, (unsigned)tiles, tma ? samp : nullptr, st);
   }
-  rc = launch_status("tile_sort_keys64");
+  int rc = launch_status("tile_sort_keys64");
   for (int pass = 0; rc == NSORT_OK && pass < p.merge_passes; ++pass) {
     const int64_t run = (int64_t)p.sort_tile << pass;
     const bool last = pass == p.merge_passes - 1;
@@ -1952,22 +1945,24 @@ int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void 
   return rc;
 }
 
+int sort_keys64_impl(const uint64_t *in, uint64_t *out, int64_t n, int dt, void *tmp,
+                     cudaStream_t st) {
+  const Plan p = make_plan(NSORT_KIND_KEYS, (uint64_t)n, dt);
+  if (p.merge_passes == 0) {
+    TraceScope tr(TK_TILE_SORT_KEYS64, st);
+    small_sort_keys64(in, out, (int)n, dt, st);
+    return launch_status("small_sort_keys64");
+  }
+  bool sorted = false;
+  const int rc = radix_sort_keys64(p, &sorted, in, out, dt, tmp, st);
+  return sorted || rc != NSORT_OK ? rc : merge_sort_keys64(p, in, out, dt, tmp, st);
+}
+
 // ---- the sorts ------------------------------------------------------------
 
-int sort_keys_impl(const uint32_t *in, uint32_t *out, int64_t n, int dt, void *tmp,
-                   cudaStream_t st) {
-  const Plan p = make_plan(NSORT_KIND_KEYS, (uint64_t)n);
-  if (p.merge_passes == 0) {
-    TraceScope tr(TK_TILE_SORT_KEYS, st);
-    small_sort_keys(in, out, (int)n, dt, st);
-    return launch_status("small_sort_keys");
-  }
-  int rc = NSORT_OK;
-  if (p.merge4_passes == 0) {
-    bool sorted = false;
-    rc = radix_sort_keys(p, &sorted, in, out, dt, tmp, st);
-    if (sorted || rc != NSORT_OK) return rc;
-  }
+static int merge_sort_keys(const Plan &p, const uint32_t *in, uint32_t *out, int dt, void *tmp,
+                           cudaStream_t st) {
+  const int64_t n = p.n;
   char *t = static_cast<char *>(tmp);
   uint32_t *bufs[2] = {out, reinterpret_cast<uint32_t *>(t + p.keys_off)};
   int64_t *split = reinterpret_cast<int64_t *>(t + p.split_off);
@@ -1989,7 +1984,7 @@ int sort_keys_impl(const uint32_t *in, uint32_t *out, int64_t n, int dt, void *t
     TraceScope tr(TK_TILE_SORT_KEYS, st);
     launch_tile_sort_keys(in, bufs[cur], n, dt, (unsigned)tiles, tma ? samp : nullptr, st);
   }
-  rc = launch_status("tile_sort_keys");
+  int rc = launch_status("tile_sort_keys");
   int64_t run = p.sort_tile;
   for (int pass = 0; rc == NSORT_OK && pass < npass; ++pass) {
     const bool last = pass == npass - 1;
@@ -2027,25 +2022,31 @@ int sort_keys_impl(const uint32_t *in, uint32_t *out, int64_t n, int dt, void *t
   return rc;
 }
 
-// Stable pairs with payload word V.  64-bit payloads take no staged-load
-// fallback: their outputs must be 16-byte aligned (the C ABI checks).
-template <typename V>
-static int sort_pairs_typed(const uint32_t *kin, const V *vin, uint32_t *kout, V *vout, int64_t n,
-                            int dt, void *tmp, cudaStream_t st) {
-  constexpr bool V64 = sizeof(V) == 8;
-  const Plan p = make_plan(V64 ? NSORT_KIND_PAIRS64 : NSORT_KIND_PAIRS, (uint64_t)n);
+int sort_keys_impl(const uint32_t *in, uint32_t *out, int64_t n, int dt, void *tmp,
+                   cudaStream_t st) {
+  const Plan p = make_plan(NSORT_KIND_KEYS, (uint64_t)n);
   if (p.merge_passes == 0) {
-    TraceScope tr(TK_TILE_SORT_PAIRS, st);
-    if constexpr (V64) small_sort_pairs64(kin, vin, kout, vout, (int)n, dt, st);
-    else small_sort_pairs(kin, vin, kout, vout, (int)n, dt, st);
-    return launch_status("small_sort_pairs");
+    TraceScope tr(TK_TILE_SORT_KEYS, st);
+    small_sort_keys(in, out, (int)n, dt, st);
+    return launch_status("small_sort_keys");
   }
-  bool sorted = false;
-  int rc;
-  if constexpr (V64) rc = radix_sort_pairs64(p, &sorted, kin, vin, kout, vout, dt, tmp, st);
-  else rc = radix_sort_pairs(p, &sorted, kin, vin, kout, vout, dt, tmp, st);
-  if (sorted || rc != NSORT_OK) return rc;
-  rc = ensure_pairs_smem_attr<V>();
+  if (p.merge4_passes == 0) {
+    bool sorted = false;
+    const int rc = radix_sort_keys(p, &sorted, in, out, dt, tmp, st);
+    if (sorted || rc != NSORT_OK) return rc;
+  }
+  return merge_sort_keys(p, in, out, dt, tmp, st);
+}
+
+// Stable pairs with payload word V, by the plan's merge passes.  64-bit
+// payloads take no staged-load fallback: their outputs must be 16-byte aligned
+// (the C ABI checks).
+template <typename V>
+static int merge_sort_pairs(const Plan &p, const uint32_t *kin, const V *vin, uint32_t *kout,
+                            V *vout, int dt, void *tmp, cudaStream_t st) {
+  constexpr bool V64 = sizeof(V) == 8;
+  const int64_t n = p.n;
+  int rc = ensure_pairs_smem_attr<V>();
   if (rc != NSORT_OK) return rc;
   char *t = static_cast<char *>(tmp);
   uint32_t *kb[2] = {kout, reinterpret_cast<uint32_t *>(t + p.keys_off)};
@@ -2088,6 +2089,24 @@ static int sort_pairs_typed(const uint32_t *kin, const V *vin, uint32_t *kout, V
     cur ^= 1;
   }
   return rc;
+}
+
+template <typename V>
+static int sort_pairs_typed(const uint32_t *kin, const V *vin, uint32_t *kout, V *vout, int64_t n,
+                            int dt, void *tmp, cudaStream_t st) {
+  constexpr bool V64 = sizeof(V) == 8;
+  const Plan p = make_plan(V64 ? NSORT_KIND_PAIRS64 : NSORT_KIND_PAIRS, (uint64_t)n);
+  if (p.merge_passes == 0) {
+    TraceScope tr(TK_TILE_SORT_PAIRS, st);
+    if constexpr (V64) small_sort_pairs64(kin, vin, kout, vout, (int)n, dt, st);
+    else small_sort_pairs(kin, vin, kout, vout, (int)n, dt, st);
+    return launch_status("small_sort_pairs");
+  }
+  bool sorted = false;
+  int rc;
+  if constexpr (V64) rc = radix_sort_pairs64(p, &sorted, kin, vin, kout, vout, dt, tmp, st);
+  else rc = radix_sort_pairs(p, &sorted, kin, vin, kout, vout, dt, tmp, st);
+  return sorted || rc != NSORT_OK ? rc : merge_sort_pairs(p, kin, vin, kout, vout, dt, tmp, st);
 }
 
 int sort_pairs_impl(const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout,
@@ -2569,6 +2588,36 @@ extern "C" int nsort_pairs64(const void *d_keys_in, const uint64_t *d_vals_in, v
   return sort_pairs64_impl(static_cast<const uint32_t *>(d_keys_in), d_vals_in,
                            static_cast<uint32_t *>(d_keys_out), d_vals_out, (int64_t)n, dtype,
                            d_tmp, static_cast<cudaStream_t>(stream));
+}
+
+extern "C" int nsort_testing_merge_sort(int kind, const void *d_keys_in, const void *d_vals_in,
+                                        void *d_keys_out, void *d_vals_out, uint64_t n, int dtype,
+                                        void *d_tmp, size_t tmp_bytes, void *stream) {
+  if (kind != NSORT_KIND_KEYS && kind != NSORT_KIND_PAIRS && kind != NSORT_KIND_PAIRS64)
+    return NSORT_EINVAL;
+  const int rc = check_common(d_keys_in, d_keys_out, n, dtype, d_tmp, tmp_bytes, kind);
+  if (rc != NSORT_OK) return rc;
+  const Plan p = make_plan(kind, n, is_wide(dtype) ? dtype : 0);
+  if (p.merge_passes == 0) return NSORT_EINVAL;   // (no scratch either)
+  const uintptr_t vals =
+      reinterpret_cast<uintptr_t>(d_vals_in) | reinterpret_cast<uintptr_t>(d_vals_out);
+  const uintptr_t outs =
+      reinterpret_cast<uintptr_t>(d_keys_out) | reinterpret_cast<uintptr_t>(d_vals_out);
+  if (kind != NSORT_KIND_KEYS && (!d_vals_in || !d_vals_out || (vals & 3))) return NSORT_EINVAL;
+  if (kind == NSORT_KIND_PAIRS64 && ((vals & 7) || (outs & 15))) return NSORT_EINVAL;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const uint32_t *kin = static_cast<const uint32_t *>(d_keys_in);
+  uint32_t *kout = static_cast<uint32_t *>(d_keys_out);
+  if (kind == NSORT_KIND_PAIRS)
+    return merge_sort_pairs(p, kin, static_cast<const uint32_t *>(d_vals_in), kout,
+                            static_cast<uint32_t *>(d_vals_out), dtype, d_tmp, st);
+  if (kind == NSORT_KIND_PAIRS64)
+    return merge_sort_pairs(p, kin, static_cast<const uint64_t *>(d_vals_in), kout,
+                            static_cast<uint64_t *>(d_vals_out), dtype, d_tmp, st);
+  if (is_wide(dtype))
+    return merge_sort_keys64(p, static_cast<const uint64_t *>(d_keys_in),
+                             static_cast<uint64_t *>(d_keys_out), dtype, d_tmp, st);
+  return merge_sort_keys(p, kin, kout, dtype, d_tmp, st);
 }
 
 extern "C" const char *nsort_status_string(int status) {

@@ -128,6 +128,8 @@ def _load():
         lib.nsort_selftest_wait.restype = i32
         lib.nsort_selftest_digit_waits.argtypes = [i32, vp, sz, ctypes.c_uint32, vp]
         lib.nsort_selftest_digit_waits.restype = i32
+        lib.nsort_testing_merge_sort.argtypes = [i32, vp, vp, vp, vp, u64, i32, vp, sz, vp]
+        lib.nsort_testing_merge_sort.restype = i32
         lib.nsort_testing_set_four_way_min.argtypes = [u64]
         lib.nsort_testing_set_four_way_min.restype = u64
         lib.nsort_keys_noalloc.argtypes = [vp, vp, u64, i32, vp]
@@ -400,6 +402,14 @@ def nsort_selftest_digit_waits(which: int, tmp, limit_us: int, stream=None) -> i
     counts that never come."""
     return _load().nsort_selftest_digit_waits(which, _ptr(tmp), tmp.numel() * tmp.element_size(),
                                               limit_us, _stream(stream))
+
+
+def nsort_testing_merge_sort(kind: int, keys_in, vals_in, keys_out, vals_out, n: int, dtype: int,
+                             tmp, tmp_bytes: int, stream=None) -> int:
+    """A plain sort by the plan's merge passes, whatever its size (test hook)."""
+    return _load().nsort_testing_merge_sort(kind, _ptr(keys_in), _ptr(vals_in), _ptr(keys_out),
+                                            _ptr(vals_out), n, dtype, _ptr(tmp), tmp_bytes,
+                                            _stream(stream))
 
 
 def nsort_testing_set_four_way_min(min_keys: int) -> int:
