@@ -285,7 +285,7 @@ int nsort_keys_noalloc_status(void *stream);
  * A context owns a scheduler thread, a pool of CUDA streams and a device
  * memory budget.  Requests (device-resident inputs and outputs owned by the
  * caller) are admitted as soon as a stream slot and budget for their scratch
- * are free; small requests are co-batched into one segmented launch;
+ * are free; small requests that wait are co-batched into one segmented launch;
  * admitted requests overlap on the device, except that requests of 2^22
  * keys or more (each fills the GPU) run one at a time, and while one runs
  * smaller requests are admitted ahead of the next.  Each result is bit-identical to
@@ -308,7 +308,10 @@ typedef struct {
     double t_admit;    /* scratch reserved, work enqueued */
     double t_done;     /* completion observed by the scheduler */
     int status;        /* nsort_status of the request */
-    int batched;       /* 1 when co-batched into a segmented launch */
+    int batched;       /* 1 when admitted as a small request (n <= batch_max_keys):
+                        * in one segmented launch with the requests admitted with
+                        * it (they share t_admit), or by the plain call when there
+                        * are none */
 } nsort_timing;
 
 /* device: CUDA ordinal.  mem_budget_bytes: size of the scratch arena the
