@@ -1519,12 +1519,20 @@ static int64_t merge4_tiles(int64_t n, int64_t run, int64_t *tpg_out, int64_t *g
   return tiles;
 }
 
-// Boundary records of the four-way passes of a plan (the most any pass
-// needs: the first four-way pass has the shortest runs).
+// Boundary records of the four-way passes of a plan, the first one over runs
+// of run0 keys: the most any pass needs.  A pass has tpg + 1 records for every
+// group, also for a partial last one, so that the first pass, with the
+// shortest runs, needs the most only if the later ones' groups are full (2^22 + 9
+// keys: 1089 records in the first, 2049 in the last).
 static int64_t merge4_records(int64_t n, int64_t run0) {
-  int64_t tpg = 0, groups = 0;
-  merge4_tiles(n, run0, &tpg, &groups);
-  return groups * (tpg + 1);
+  int64_t most = 0;
+  for (int64_t run = run0; run < n; run *= 4) {
+    int64_t tpg = 0, groups = 0;
+    merge4_tiles(n, run, &tpg, &groups);
+    const int64_t records = groups * (tpg + 1);
+    most = most > records ? most : records;
+  }
+  return most;
 }
 
 Plan make_plan(int kind, uint64_t n, int dtype) {

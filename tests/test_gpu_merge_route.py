@@ -109,12 +109,15 @@ def test_two_way_and_four_way_agree(ns):
     for setting, name in ((ns.FOUR_WAY_NEVER, "merge_keys"), (0, "merge4_keys")):
         prev = ns.nsort_testing_set_four_way_min(setting)
         try:
-            tmp, out = ns.scratch(ns.KIND_KEYS, n), torch.empty_like(x)
+            need, out = ns.nsort_temp_bytes(ns.KIND_KEYS, n), torch.empty_like(x)
+            tmp = torch.full((need + (1 << 17),), 0x5A, dtype=torch.uint8, device="cuda")
             ns.nsort_trace_enable(True)
             assert ns.nsort_testing_merge_sort(ns.KIND_KEYS, x, None, out, None, n, ns.F32, tmp,
-                                               tmp.numel()) == ns.OK
+                                               need) == ns.OK
             assert name in route(ns.nsort_trace_read())
             ns.nsort_trace_enable(False)
+            assert ns.nsort_device_status(tmp) == ns.OK
+            assert bool((tmp[need:] == 0x5A).all()), "wrote past the scratch"
         finally:
             ns.nsort_testing_set_four_way_min(prev)
         outs.append(out.cpu().numpy().view(np.uint32))
