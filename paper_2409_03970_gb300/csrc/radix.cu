@@ -419,8 +419,10 @@ struct DigitTile {
 
   // Ranks the thread's keys I0 .. I1 - 1 and stages them in order (the digits
   // are extracted anew: kept from the counting they would cost a register
-  // per key).
-  template <int I0 = 0, int I1 = IPT>
+  // per key).  FREE_PARTIAL: a partial tile's warps may rank in free order too
+  // (64-bit look-back passes, with one such tile in hundreds, leave that out:
+  // 2^27 int64 keys 4.89 -> 4.86 ms, 4.0e6 206.7 -> 204.5 us).
+  template <int I0 = 0, int I1 = IPT, bool FREE_PARTIAL = true>
   __device__ __forceinline__ void rank(const K (&r)[IPT], uint32_t (&pos2)[NPOS]) {
     asm volatile("" : "+r"(sel));
     uint32_t *mine = my_counters();
@@ -444,8 +446,8 @@ struct DigitTile {
       // the keys of this warp may be order-free even if the tile's are not
       const K f = __shfl_sync(0xffffffffu, r[0], lane & 16) & low;
       const K l = __shfl_sync(0xffffffffu, r[IPT - 1], lane | 15) & low;
-      if (__all_sync(0xffffffffu, f == l)) {
-        if (count == TILE) {
+      if ((FREE_PARTIAL || count == TILE) && __all_sync(0xffffffffu, f == l)) {
+        if (!FREE_PARTIAL || count == TILE) {
 #pragma unroll
           for (int i = I0; i < I1; ++i)
             stage[staged(atomicAdd(mine + 2 * digit(r[i]), 1u << 16) >> 16)] = r[i];
@@ -614,7 +616,7 @@ __device__ __forceinline__ uint32_t load_of_cta(const uint32_t *p, uint32_t c) {
 // before it runs and well within L2: 2^28 keys take 3.00 ms without, 2.96 with
 // 20 tiles, 2.80 with 50, 2.79 with 76 to 304, 2.93 with 608 (40 MB ahead, in
 // L2 beside the scattered writes).
-constexpr uint32_t AHEAD = 76;   // tiles: a quarter of those that run at once
+constexpr uint32_t AHEAD = 76;   // tiles: a quarter of the 304 that run at once on 152 SMs
 template <typename K, typename V, int IPT, bool FIRST, bool LAST, bool WAVE, int CL = 1>
 __global__ void __launch_bounds__(NT, 2) radix_pass_kernel(
     const K *src, const V *vsrc, K *__restrict__ dst, V *__restrict__ vdst, uint32_t n, int shift,
@@ -761,7 +763,7 @@ __global__ void __launch_bounds__(NT, 2) radix_pass_kernel(
     if (!(tid & 1)) sh.gbase[d] = excl - tbase;
     if (excl + total > n + (d == BINS - 1 ? T::TILE - count : 0)) flags |= 1;
   } else {
-    t.rank(r, pos2);
+    t.template rank<0, IPT, sizeof(K) == 4>(r, pos2);
     // where the tile's keys go
     uint32_t excl = 0;
     if (tile == 0) {   // the digit's first position: all keys of smaller digits
@@ -1110,7 +1112,11 @@ int radix_sort_typed(const Plan &p, bool *sorted, const K *in, const V *vin, K *
   *sorted = false;
   if (p.n >= (int64_t(1) << 30)) return NSORT_OK;   // (counts take 30 bits)
   // 64-bit keys take eight passes, which the merge passes beat, on sorted keys
-  // at least, outside two ranges.  int64, uniform / sorted, merges -> digits:
+  // at least, outside two ranges; beyond them digits are 2-4% slower on sorted
+  // keys up to 2.0e6 and 10-18% faster on others, which the host can't tell
+  // apart.  The lines lie where they do on 152 SMs: 5 << 17 is 0.70 of a
+  // 6144-key tile on each of them, 9 << 17 0.95 of an 8192-key one.  int64,
+  // uniform / sorted, merges -> digits:
   //   5.0e5: 60 / 55 -> 64 / 64;  6.6e5 (5 << 17): 77 / 69 -> 64 / 64;
   //   9.3e5: 81 / 72 -> 70 / 70;  then a larger tile: 9.5e5: 83 / 73 -> 80 / 79,
   //   1.1e6: 92 / 81 -> 82 / 82;  1.18e6 (9 << 17): 106 / 90 -> 84 / 83;

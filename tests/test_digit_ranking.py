@@ -20,10 +20,11 @@ def padding_takes_part():
     """Whether a free-order atomic of a partial tile is done for padding too."""
     with open(os.path.join(ROOT, "paper_2409_03970_gb300", "csrc", "radix.cu")) as f:
         text = re.sub(r"//[^\n]*|#pragma[^\n]*", "", f.read())
-    branch = re.search(r"if \(__all_sync\(0xffffffffu, f == l\)\) \{(.*?)\n      \} else \{", text,
+    branch = re.search(r"__all_sync\(0xffffffffu, f == l\)\) \{(.*?)\n      \} else \{", text,
                        re.S).group(1)
     full, _, partial = branch.partition("} else {")
-    return not (re.match(r"\s*if \(count == TILE\) \{", full) and
+    return not (re.match(r"\s*if \(!FREE_PARTIAL \|\| count == TILE\) \{", full) and
+                "(FREE_PARTIAL || count == TILE) && __all_sync" in text and
                 re.search(r"if \(e0 \+ 16 \* i < count\)\s*stage\[", partial))
 
 
