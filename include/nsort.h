@@ -89,14 +89,16 @@ typedef enum {
  * keys (and values), plus the per-tile merge-path splitters. */
 size_t nsort_temp_bytes(int kind, uint64_t n, uint64_t nseg, int dtype);
 
-/* Number of passes over the data for a plain sort of n 32-bit keys (kind
+/* Number of passes over the data for a merge sort of n 32-bit keys (kind
  * KEYS or PAIRS): one tile sort plus ceil(log2(ceil(n / tile))) global merge
- * passes.  Writes the tile sizes through the non-NULL pointers.  Used to
- * compute the algorithmic bytes of a sort (passes x 2 x element bytes x n).
- * This is the plan of the merge sort; most sorts of more than a tile (of
- * 64-bit keys: of more than 655,360, but for some around a million) are done
- * in as many stable passes over the array as a key has bytes instead, with the
- * same result and the same scratch. */
+ * passes.  Writes the tile sizes through the non-NULL pointers.  This plan
+ * sizes the scratch of every plain sort and gives the algorithmic bytes of
+ * one that merges (passes x 2 x element bytes x n).  Most sorts of more than
+ * a tile and fewer than 2^30 elements (of 64-bit keys: of 655,360 or more, but
+ * for some around a million) are done in as many stable passes over the array
+ * as a key has bytes instead, after one read of the keys, with the same result
+ * and scratch; which way a sort went is in its trace (radix_pass, radix_cluster
+ * or merge_...). */
 int nsort_plan(int kind, uint64_t n, int *passes, int *sort_tile, int *merge_tile);
 
 /* nsort_plan for keys of `dtype`: 64-bit dtypes (kind KEYS only) sort

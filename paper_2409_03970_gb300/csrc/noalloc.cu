@@ -30,9 +30,11 @@ namespace {
 
 // Scratch of a plain key sort of NSORT_NOALLOC_MAX_KEYS keys, laid out as
 // nsort_keys lays out its scratch: the device status word, one ping-pong
-// copy of the keys, one int64 merge-path splitter per merge tile (sized for
-// merge tiles of 256 keys or more) and every 64th key of a pass's output;
-// each part rounded up to 256 bytes (about 4.1 MiB in all).
+// copy of the keys, and what a merge sort of them would take for splitters (an
+// int64 per merge tile, sized for merge tiles of 256 keys or more) and samples
+// (every 64th key), where the digit passes that sort these sizes put their
+// histograms, tickets and tile counts; each part rounded up to 256 bytes (about
+// 4.1 MiB in all).
 constexpr size_t kStatusBytes = 256;
 constexpr size_t kKeysBytes = size_t(NSORT_NOALLOC_MAX_KEYS) * 4;
 constexpr size_t kSplitBytes = ((NSORT_NOALLOC_MAX_KEYS / 256 + 2) * 8 + 255) / 256 * 256;
@@ -99,10 +101,10 @@ extern "C" int nsort_keys_noalloc(const void *d_keys_in, void *d_keys_out, uint6
   if (rc != NSORT_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // The status word (the array's first bytes) starts every call at
-  // NSORT_OK, also for sorts without merge passes, which never write it:
+  // NSORT_OK, also for sorts of one tile, which never write it:
   // nsort_keys_noalloc_status then always reports this call.  Nothing else
-  // in the scratch has to start at zero: the tile sort writes the whole key
-  // buffer and every pass writes its splitters before reading them.
+  // in the scratch has to start at zero: every pass writes the whole key buffer
+  // that the next one reads, and a sort sets its counters itself.
   if (cudaMemsetAsync(scratch, 0, sizeof(int), st) != cudaSuccess) {
     set_last_error(std::string("nsort_keys_noalloc: cudaMemsetAsync: ") +
                    cudaGetErrorString(cudaGetLastError()));

@@ -594,13 +594,13 @@ __device__ __forceinline__ uint32_t load_of_cta(const uint32_t *p, uint32_t c) {
 // which leaves room in the scratch for short tiles: the CTAs exchange their
 // counts through distributed shared memory.  A wave pass is alive while the
 // pass before it still writes (pdl_trigger), so it reads what that one and the
-// histogram kernel write as such; a look-back pass starts when its
-// predecessor has ended, and may take the read-only path.
+// histogram kernel write by loads for that (Writer); a look-back pass starts
+// when its predecessor has ended, and may take the read-only path.
 //
 // What bounds it (ncu at 2^26 uniform u32 keys): the LSU data pipe in the
 // stable passes (20-22 shared-memory wavefronts for 32 keys beside the
-// scattered stores, 83-85% of the pipe's peak; 190 and 207 us), and in the
-// free-order passes (11 wavefronts, 67-70%; 147-151 us) the latency of the
+// scattered stores, 82-85% of the pipe's peak; 193 and 207 us), and in the
+// free-order passes (11 wavefronts, 67-69%; 149-151 us) the latency of the
 // phases of the two tiles an SM holds at a time.  A pass
 // over 2^28 keys takes 0.65 ms on average, 3.3 TB/s of keys; 2^28 keys sort
 // in 2.78 ms against 6.42 ms by merge passes, 2^27 f32 pairs in 2.43 against
