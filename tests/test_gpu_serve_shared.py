@@ -45,15 +45,15 @@ def serve(ns, reqs, head_keys):
 
 
 def test_requests_that_wait_share_a_launch(ns):
-    """40 requests wait behind 2^28 keys (2.8 ms; they take less than 1 to submit)."""
-    reqs = [inputs.keys(1000 + 997 * i, "u32", "uniform", seed=i) for i in range(40)]
-    timings, launches = serve(ns, reqs, 1 << 28)
+    """24 requests wait behind 2^29 keys (5.6 ms; they take some 0.3 to submit)."""
+    reqs = [inputs.keys(1000 + 997 * i, "u32", "uniform", seed=i) for i in range(24)]
+    timings, launches = serve(ns, reqs, 1 << 29)
     assert all(t["batched"] for t in timings)
     assert len({t["t_admit"] for t in timings}) == 1
     assert launches["segmented_sort"] == 1 and "radix_cluster" not in launches
 
 
 def test_a_request_alone_takes_the_plain_call(ns):
-    timings, launches = serve(ns, [inputs.keys(40_000, "u32", "uniform", seed=1)], 1 << 28)
+    timings, launches = serve(ns, [inputs.keys(40_000, "u32", "uniform", seed=1)], 1 << 29)
     assert timings[0]["batched"]
     assert "segmented_sort" not in launches and launches["radix_cluster"] == 1
